@@ -36,12 +36,14 @@
 // the x-boundary cells sit at lead-1 and lead+nx.  Planes 0 and nz+1, rows 0
 // and ny+1 and the x-boundary cells hold the Dirichlet zeros in both buffers
 // and are never written after creation, so a pointer swap keeps them intact.
+#include <algorithm>
 #include <cmath>
 #include <vector>
 #include <cstdlib>
 #include <new>
 #include <type_traits>
 
+#include "gridbar.cuh"
 #include "heat_common.cuh"
 #include "tma.cuh"
 
@@ -295,6 +297,7 @@ struct hs_heat {
     long long R;       // FIXED64: r 2^64
     uint32_t flags;
     cudaStream_t stream;
+    void* arena;       // the handle's device allocation: err, fx, msync and, if it owns them, buf[]
     void* buf[2];
     bool owns_buf;     // false: buf[] are the caller's dev_buf0/dev_buf1
     FxState* fx;       // FIXED64 only
@@ -318,6 +321,7 @@ struct hs_heat {
     // and joined back before the next one (ev_join).  Null: one stream.
     cudaStream_t bstream;
     cudaEvent_t ev_fork, ev_join;
+    void* msync;           // grid-barrier memory of the multi-step kernel; null: the handle does not use it
     // heat_time_interior: event pairs around the Interior launches of heat_step
     bool timing;
     std::vector<cudaEvent_t> tev;   // 2 per recorded launch, reused
@@ -325,6 +329,11 @@ struct hs_heat {
 };
 
 namespace {
+
+// Layout of the words at the start of a handle's allocation.
+constexpr size_t kHeatFxOffset = 128, kHeatBarOffset = 256;
+constexpr size_t kHeatStateBytes = (kHeatBarOffset + kGridBarBytes + 255) / 256 * 256;
+static_assert(sizeof(FxState) <= kHeatBarOffset - kHeatFxOffset, "the per-step state fits its slot");
 
 constexpr int64_t kForkMinPoints = (int64_t)1 << 22;
 constexpr size_t kMaxTimedLaunches = 8192;   // event pairs a handle keeps for heat_interior_time
@@ -630,6 +639,47 @@ int pick_kc_stream(const HeatGeom& g, int arith)
     return (int)kc;
 }
 
+// Whether heat_step advances this handle with the multi-step kernel: grids
+// below 2^22 points, 2^23 in FP32, unless the caller asked for another schedule
+// or depth.  Measured per step, Interior + Boundary launches (FP32: the blocked
+// pass) against it: 64^3 FP64 14.4 / 3.8 us, FP32 9.3 / 2.6; 128^3 FP64 18.5 /
+// 13.5, FP32 10.3 / 5.9; 160^3 FP64 27.6 / 25.5, FIXED64 24.8 / 20.0, FP32 13.4
+// / 7.9; 192^3 FP64 32.8 / 35.6, FIXED64 28.8 / 29.1, FP32 13.4 / 10.8; 224^3
+// FP32 20.6 / 21.0.
+bool use_multi(const hs_heat_desc* d, const hs_heat* h)
+{
+    if (d->flags & (HS_SCHED_FULL | HS_VARKAPPA)) return false;
+    if (h->arith != A_F32 && h->arith != A_FX64 && h->arith != A_F64_XS) return false;
+    if (d->tdepth > 1) return false;   // the caller asked for temporal blocking
+    const int64_t npts = (int64_t)h->g.nx * h->g.ny * h->g.nz;
+    return npts < ((int64_t)1 << (h->arith == A_F32 ? 23 : 22));
+}
+
+// n_steps steps in one launch of the multi-step kernel.
+int multi_steps(hs_heat* h, int n_steps)
+{
+    MultiCall c;
+    c.arith = h->arith;
+    c.buf[0] = h->buf[0];
+    c.buf[1] = h->buf[1];
+    c.cur = h->cur;
+    c.g = &h->g;
+    c.r = h->r;
+    c.R = h->R;
+    c.fx = h->fx;
+    c.m3 = (int)(h->fxseq % 3);
+    c.steps = n_steps;
+    c.sync = h->msync;
+    c.err = h->err;
+    c.stream = h->stream;
+    const int rc = multi_launch(c);
+    if (rc != HS_OK) return rc;
+    h->cur = (int)((h->cur + n_steps) & 1);
+    h->steps += n_steps;
+    h->fxseq += n_steps;
+    return HS_OK;
+}
+
 // One pass of L steps with the temporally blocked kernel.
 int tb_pass(hs_heat* h, int L)
 {
@@ -822,34 +872,30 @@ int heat_create(hs_heat_t* out, const hs_heat_desc* desc)
         return rc;
     }
     h->owns_buf = !desc->dev_buf0;
-    for (int b = 0; b < 2; ++b) {
-        cudaError_t e = cudaSuccess;
-        if (h->owns_buf) {
-            e = dev_alloc(&h->buf[b], bytes, h->stream);
-        } else {
-            h->buf[b] = b == 0 ? desc->dev_buf0 : desc->dev_buf1;
-        }
-        if (e != cudaSuccess) {
-            h->buf[b] = nullptr;
-            rc = cuda_fail(e, "heat_create: device allocation");
-            heat_destroy(h);
-            return rc;
-        }
-        e = cudaMemsetAsync(h->buf[b], 0, bytes, h->stream);
-        if (e != cudaSuccess) {
-            rc = cuda_fail(e, "heat_create: cudaMemsetAsync");
-            heat_destroy(h);
-            return rc;
-        }
+    // one allocation holds the handle's words (error word, per-step state, grid
+    // barrier) and, unless the caller owns them, the two buffers
+    const size_t fbytes = (bytes + 255) & ~(size_t)255;
+    const size_t total = kHeatStateBytes + (h->owns_buf ? 2 * fbytes : 0);
+    cudaError_t ea = dev_alloc(&h->arena, total, h->stream);
+    if (ea != cudaSuccess) {
+        h->arena = nullptr;
+        rc = cuda_fail(ea, "heat_create: device allocation");
+        heat_destroy(h);
+        return rc;
     }
-    {
-        cudaError_t e = dev_alloc((void**)&h->err, sizeof(int), h->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(h->err, 0, sizeof(int), h->stream);
-        if (e != cudaSuccess) {
-            rc = cuda_fail(e, "heat_create: error word");
-            heat_destroy(h);
-            return rc;
-        }
+    char* const base = (char*)h->arena;
+    h->err = (int*)base;
+    FxState* const fx_state = (FxState*)(base + kHeatFxOffset);
+    if (use_multi(desc, h)) h->msync = base + kHeatBarOffset;
+    h->buf[0] = h->owns_buf ? (void*)(base + kHeatStateBytes) : desc->dev_buf0;
+    h->buf[1] = h->owns_buf ? (void*)(base + kHeatStateBytes + fbytes) : desc->dev_buf1;
+    ea = cudaMemsetAsync(h->arena, 0, total, h->stream);
+    for (int b = 0; b < 2 && !h->owns_buf && ea == cudaSuccess; ++b)
+        ea = cudaMemsetAsync(h->buf[b], 0, bytes, h->stream);
+    if (ea != cudaSuccess) {
+        rc = cuda_fail(ea, "heat_create: cudaMemsetAsync");
+        heat_destroy(h);
+        return rc;
     }
     {
         const CUtensorMapDataType dt = h->arith == A_FX64   ? CU_TENSOR_MAP_DATA_TYPE_INT64
@@ -889,15 +935,7 @@ int heat_create(hs_heat_t* out, const hs_heat_desc* desc)
             }
         }
     }
-    if (h->arith == A_FX64 || h->arith == A_F64_XS) {
-        cudaError_t e = dev_alloc((void**)&h->fx, sizeof(FxState), h->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(h->fx, 0, sizeof(FxState), h->stream);
-        if (e != cudaSuccess) {
-            rc = cuda_fail(e, "heat_create: fixed-point state");
-            heat_destroy(h);
-            return rc;
-        }
-    }
+    if (h->arith == A_FX64 || h->arith == A_F64_XS) h->fx = fx_state;
     if (h->flags & HS_VARKAPPA) {
         const size_t bytes = (size_t)h->g.total * h->elem;
         // FP64 keeps the three face sums of kappa, FP32 kappa itself
@@ -946,15 +984,7 @@ int heat_create(hs_heat_t* out, const hs_heat_desc* desc)
         }
         // FP64 with every face sum of kappa in [1, 2): the exact-sum form,
         // which tracks the field's largest exponent step by step
-        if (h->dtype == HS_F64 && face_off == 0) {
-            e = dev_alloc((void**)&h->fx, sizeof(FxState), h->stream);
-            if (e == cudaSuccess) e = cudaMemsetAsync(h->fx, 0, sizeof(FxState), h->stream);
-            if (e != cudaSuccess) {
-                rc = cuda_fail(e, "heat_create: exact-sum state");
-                heat_destroy(h);
-                return rc;
-            }
-        }
+        if (h->dtype == HS_F64 && face_off == 0) h->fx = fx_state;
     }
     // A Boundary kernel beside the Interior one pays for its extra API calls
     // once the Interior kernel takes tens of microseconds (2^22 points and up).
@@ -1033,6 +1063,15 @@ int heat_step(hs_heat_t h, int64_t n_steps)
 {
     if (!h) return fail(HS_EINVAL, "heat_step: NULL handle");
     if (n_steps < 0) return fail(HS_EINVAL, "heat_step: n_steps = %lld < 0", (long long)n_steps);
+    if (h->msync && !h->timing) {
+        while (n_steps > 0) {
+            const int part = (int)std::min<int64_t>(n_steps, (int64_t)1 << 20);
+            const int rc = multi_steps(h, part);
+            if (rc != HS_OK) return rc;
+            n_steps -= part;
+        }
+        return HS_OK;
+    }
     if (h->tdepth > 1) {
         // passes of tdepth steps, then the remainder in the largest built depths
         int64_t left = n_steps;
@@ -1192,7 +1231,7 @@ int heat_destroy(hs_heat_t h)
 {
     if (!h) return HS_OK;
     int rc = HS_OK;
-    if (h->buf[0] || h->buf[1]) {
+    if (h->arena) {
         cudaError_t e = cudaStreamSynchronize(h->stream);
         if (e != cudaSuccess) rc = cuda_fail(e, "heat_destroy: stream synchronize");
     }
@@ -1204,10 +1243,7 @@ int heat_destroy(hs_heat_t h)
     for (cudaEvent_t e : h->tev) (void)cudaEventDestroy(e);
     if (h->ev_fork) (void)cudaEventDestroy(h->ev_fork);
     if (h->ev_join) (void)cudaEventDestroy(h->ev_join);
-    if (h->owns_buf)
-        for (int b = 0; b < 2; ++b) dev_free(h->buf[b], h->stream);
-    dev_free(h->fx, h->stream);
-    dev_free(h->err, h->stream);
+    dev_free(h->arena, h->stream);
     dev_free(h->kap, h->stream);
     dev_free(h->fdt, h->stream);
     delete h;

@@ -329,6 +329,22 @@ struct VkCall {
 int vk_init(const VkCall& c, double dt);
 int vk_launch(const VkCall& c);
 
+// One launch of the multi-step kernel (heat_multi.cu): `steps` whole steps.
+struct MultiCall {
+    int arith;               // A_F32, A_FX64 or A_F64_XS
+    void* buf[2];
+    int cur;                 // buffer holding the field
+    const HeatGeom* g;
+    double r;
+    long long R;
+    FxState* fx;
+    int m3;
+    int steps;
+    void* sync;              // kGridBarBytes of device memory (gridbar.cuh), zeroed at creation
+    int* err;
+    cudaStream_t stream;
+};
+int multi_launch(const MultiCall& c);
 // What the batched kernel needs to know about a heat handle (heat.cu).
 struct HeatBatchView {
     HeatGeom g;
