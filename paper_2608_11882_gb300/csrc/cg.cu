@@ -17,12 +17,14 @@
 // read the stop flag on entry and return at once after convergence, so the
 // host can enqueue several iterations between convergence checks without the
 // extra ones changing anything.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
+#include <cstddef>
 #include <mutex>
 #include <new>
 
-#include "cg_common.cuh"
+#include "cg_small.cuh"
 
 namespace hcg {
 
@@ -377,11 +379,7 @@ int cg_destroy(hs_cg_t c)
     int rc = HS_OK;
     cudaError_t e = cudaStreamSynchronize(c->stream);
     if (e != cudaSuccess) rc = cuda_fail(e, "cg_destroy: stream synchronize");
-    dev_free(c->r, c->stream);
-    dev_free(c->p, c->stream);
-    dev_free(c->q, c->stream);
-    dev_free(c->partials, c->stream);
-    dev_free(c->S, c->stream);
+    dev_free(c->arena, c->stream);
     delete c->S_host;
     for (void* o : c->owned) dev_free(o, c->stream);
     if (c->mx) cg_mixed_release(c->mx, c->stream);
@@ -391,7 +389,20 @@ int cg_destroy(hs_cg_t c)
     return rc;
 }
 
-int cg_create(hs_cg_t* out, const hs_op* A, void* stream)
+}  // extern "C"
+
+namespace hcg {
+
+// Doubles of reduction partials a solve of A needs.
+size_t cg_partials(const OpDev& A, int grid)
+{
+    CgSmallSys s;
+    const size_t small = cg_small_shape(A, &s) ? 2 * (size_t)s.bricks : 0;
+    return std::max(2 * (size_t)grid, small);
+}
+
+// cg_create; need_p = false leaves out the FP64 direction (mixed precision).
+int cg_create_vectors(hs_cg_t* out, const hs_op* A, void* stream, bool need_p)
 {
     if (!out) return fail(HS_EINVAL, "cg_create: out is NULL");
     *out = nullptr;
@@ -412,11 +423,16 @@ int cg_create(hs_cg_t* out, const hs_op* A, void* stream)
             return rc;                                                       \
         }                                                                    \
     } while (0)
-    CG_ALLOC(c->r, sizeof(double) * n);
-    CG_ALLOC(c->p, sizeof(double) * n);
-    CG_ALLOC(c->q, sizeof(double) * n);
-    CG_ALLOC(c->partials, sizeof(double) * 2 * c->grid);
-    CG_ALLOC(c->S, sizeof(CgScalars));
+    auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t s_ctl = align(sizeof(CgSmallCtl)), s_part = align(sizeof(double) * cg_partials(c->A, c->grid));
+    const size_t s_vec = align(sizeof(double) * (size_t)cg_vector_len(c->A));
+    CG_ALLOC(c->arena, s_ctl + s_part + (need_p ? 3 : 2) * s_vec);
+    c->ctl = (char*)c->arena;
+    c->S = &((CgSmallCtl*)c->ctl)->S;
+    c->partials = (double*)(c->ctl + s_ctl);
+    c->r = (double*)(c->ctl + s_ctl + s_part);
+    c->q = (double*)(c->ctl + s_ctl + s_part + s_vec);
+    c->p = need_p ? (double*)(c->ctl + s_ctl + s_part + 2 * s_vec) : nullptr;
     // the host mirror of the scalars: ordinary memory (pinned memory would
     // cost a device-wide synchronisation to allocate and to free)
     c->S_host = new (std::nothrow) CgScalars();
@@ -455,6 +471,66 @@ int cg_create(hs_cg_t* out, const hs_op* A, void* stream)
     return HS_OK;
 }
 
+// What a finished FP64 solve reports (its scalars in f).
+static int cg_report(const CgScalars& f, double rtol, int32_t max_iter, hs_cg_info* info)
+{
+    const bool converged = (f.done == 1);
+    if (f.done == 2) return fail(HS_ECUDA, "cg_run: breakdown, p.q <= 0 (operator not positive definite?)");
+    if (f.done == 3) return fail(HS_ETIMEOUT, "cg_run: a bounded wait in the TMA-staged SpMV ran out");
+    if (f.done == 4)
+        return fail(HS_ECUDA, "cg_run: a bounded wait in the TMA-staged SpMV ran out and its loads in "
+                              "flight did not complete in time; treat the CUDA context as suspect");
+    if (info) {
+        info->iters = f.iters;
+        info->relres_recur = f.relres;
+        info->relres_true = f.zero_rhs ? 0.0 : sqrt(f.rr_true) / f.bnorm;
+        info->status = converged ? HS_OK : HS_ENOCONV;
+        info->refinements = 0;
+        info->reserved = 0;
+    }
+    if (!converged) {
+        set_error("cg_run: no convergence to rtol %g within %d iterations (relres %g)", rtol,
+                  max_iter, f.relres);
+        return HS_ENOCONV;
+    }
+    return HS_OK;
+}
+
+// The whole solve in one launch (cg_small.cu): b and x device vectors.
+static int cg_run_small(hs_cg* c, CgSmallSys sys, const double* b, double* x, double rtol, int32_t max_iter)
+{
+    CgSmallCtl ctl;
+    memset(&ctl, 0, sizeof(ctl));
+    CgSmallCtl* d = (CgSmallCtl*)c->ctl;
+    sys.max_iter = max_iter;
+    sys.b = b;
+    sys.x = x;
+    sys.r = c->r;
+    sys.p = c->p;
+    sys.q = c->q;
+    sys.part = c->partials;
+    sys.S = c->S;
+    ctl.sys = sys;
+    ctl.group.count = 1;
+    ctl.S.rtol = rtol;
+    HS_TRY_CUDA(cudaMemcpyAsync(d, &ctl, sizeof(ctl), cudaMemcpyHostToDevice, c->stream), "cg_run: scalar init");
+    const int rc = cg_small_launch(&d->sys, &d->group, 1, true, sys.bricks, d->bar, &d->err, c->stream);
+    if (rc != HS_OK) return rc;
+    HS_TRY_CUDA(cudaMemcpyAsync(&ctl.err, &d->err, sizeof(ctl) - offsetof(CgSmallCtl, err), cudaMemcpyDeviceToHost,
+                                c->stream),
+                "cg_run: scalar readback");
+    HS_TRY_CUDA(cudaStreamSynchronize(c->stream), "cg_run: synchronize");
+    if (ctl.err) return fail(HS_ETIMEOUT, "cg_run: a bounded wait in the small-system kernel ran out");
+    *c->S_host = ctl.S;
+    return HS_OK;
+}
+
+}  // namespace hcg
+
+extern "C" {
+
+int cg_create(hs_cg_t* out, const hs_op* A, void* stream) { return cg_create_vectors(out, A, stream, true); }
+
 int cg_run(hs_cg_t c, const void* b_in, void* x_inout, int host_buffers, double rtol,
            int32_t max_iter, hs_cg_info* info)
 {
@@ -475,6 +551,17 @@ int cg_run(hs_cg_t c, const void* b_in, void* x_inout, int host_buffers, double 
         if (rc_ != HS_OK) return rc_;
         b = c->bx_dev[0];
         x = c->bx_dev[1];
+    }
+    CgSmallSys small;
+    if (cg_small_shape(c->A, &small)) {
+        int rc_ = cg_run_small(c, small, b, x, rtol, max_iter);
+        if (rc_ != HS_OK) return rc_;
+        if (host_buffers) {
+            rc_ = copy_host(x_inout, x, vbytes, false, c->stream, "cg_run: copy of x");
+            if (rc_ != HS_OK) return rc_;
+            HS_TRY_CUDA(cudaStreamSynchronize(c->stream), "cg_run: synchronize");
+        }
+        return cg_report(*c->S_host, rtol, max_iter, info);
     }
     // device scalars: rtol, cleared flags
     CgScalars init;
@@ -550,27 +637,7 @@ int cg_run(hs_cg_t c, const void* b_in, void* x_inout, int host_buffers, double 
         if (rc_ != HS_OK) return rc_;
     }
     HS_TRY_CUDA(cudaStreamSynchronize(c->stream), "cg_run: synchronize");
-    const CgScalars f = *c->S_host;
-    const bool converged = (f.done == 1);
-    if (f.done == 2) return fail(HS_ECUDA, "cg_run: breakdown, p.q <= 0 (operator not positive definite?)");
-    if (f.done == 3) return fail(HS_ETIMEOUT, "cg_run: a bounded wait in the TMA-staged SpMV ran out");
-    if (f.done == 4)
-        return fail(HS_ECUDA, "cg_run: a bounded wait in the TMA-staged SpMV ran out and its loads in "
-                              "flight did not complete in time; treat the CUDA context as suspect");
-    if (info) {
-        info->iters = f.iters;
-        info->relres_recur = f.relres;
-        info->relres_true = f.zero_rhs ? 0.0 : sqrt(f.rr_true) / f.bnorm;
-        info->status = converged ? HS_OK : HS_ENOCONV;
-        info->refinements = 0;
-        info->reserved = 0;
-    }
-    if (!converged) {
-        set_error("cg_run: no convergence to rtol %g within %d iterations (relres %g)", rtol,
-                  max_iter, f.relres);
-        return HS_ENOCONV;
-    }
-    return HS_OK;
+    return cg_report(*c->S_host, rtol, max_iter, info);
 }
 
 int cg_solve(const hs_op* A, const void* b, void* x, double rtol, int32_t max_iter,
@@ -603,9 +670,11 @@ namespace hcg {
 
 constexpr int64_t kNoAllocMaxN = HS_NOALLOC_MAX_N;          // 2,097,152 unknowns = 128^3
 constexpr int64_t kNoAllocMaxGrid = (int64_t)kNumSMs * 8;   // the largest grid grid_for() picks
-constexpr size_t kNoAllocScalarDoubles = (sizeof(CgScalars) + sizeof(double) - 1) / sizeof(double);
-constexpr size_t kNoAllocDoubles =
-    3 * (size_t)kNoAllocMaxN + 2 * (size_t)kNoAllocMaxGrid + kNoAllocScalarDoubles;
+constexpr size_t kNoAllocCtlDoubles = (sizeof(CgSmallCtl) + 255) / 256 * 256 / sizeof(double);
+constexpr size_t kNoAllocPartials = 2 * (size_t)(kNoAllocMaxGrid > kCgSmallMaxBricks ? kNoAllocMaxGrid : kCgSmallMaxBricks);
+// n values, and the padding of odd rows of at least kCgSmallMinNx
+constexpr size_t kNoAllocVector = (size_t)(kNoAllocMaxN + kNoAllocMaxN / kCgSmallMinNx);
+constexpr size_t kNoAllocDoubles = 3 * kNoAllocVector + kNoAllocPartials + kNoAllocCtlDoubles;
 
 // About 50 MB.  Every GPU that loads this library holds it until the process exits.
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocDoubles];
@@ -654,10 +723,11 @@ int cg_solve_noalloc(const hs_op* A, const void* b, void* x, double rtol, int32_
     c.stream = (cudaStream_t)stream;
     c.grid = grid_for(c.A.n);
     c.r = base;
-    c.p = base + kNoAllocMaxN;
-    c.q = base + 2 * kNoAllocMaxN;
-    c.partials = base + 3 * kNoAllocMaxN;
-    c.S = (CgScalars*)(c.partials + 2 * kNoAllocMaxGrid);
+    c.p = base + kNoAllocVector;
+    c.q = base + 2 * kNoAllocVector;
+    c.partials = base + 3 * kNoAllocVector;
+    c.ctl = (char*)(c.partials + kNoAllocPartials);
+    c.S = &((CgSmallCtl*)c.ctl)->S;
     // cg_run clears the device scalars (stop flag, iteration count and the
     // reduction ticket, which must start at zero) before the first kernel;
     // r, p and q are written before they are read.  The copies through this

@@ -8,12 +8,13 @@
 // alone bit for bit.  Systems that have converged (or hit max_iter) stop at
 // the top of each kernel; the host reads all stop flags once per chunk of
 // iterations.
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
 #include <vector>
 
-#include "cg_common.cuh"
+#include "cg_small.cuh"
 
 namespace hcg {
 
@@ -229,15 +230,34 @@ __global__ void __launch_bounds__(kCgBlock) k_cgb_resid(const SysDev* sys, int n
 
 using namespace hcg;
 
+// Control words of the small systems' launch, uploaded whole before a run.
+struct SmallCtl {
+    unsigned long long bar[6 * kGridBarStride];
+    int32_t err;
+    int32_t pad[31];
+};
+
 struct hs_cg_batch {
     cudaStream_t stream;
     int32_t n;
+    // systems that run three kernels per iteration
+    std::vector<int32_t> big;  // their places in the batch
     int32_t total_blocks;
     bool has_mode[3];          // SpmvModes present (one SpMV kernel each)
     std::vector<SysDev> sys;   // host copy (b, x filled per run)
-    std::vector<int64_t> rows;
     SysDev* d_sys;
-    void* arena;               // r, p, q, partials, scalars of all systems
+    // small matrix-free systems, solved whole in one launch (cg_small.cu)
+    std::vector<int32_t> small;         // their places in the batch, group after group
+    std::vector<CgSmallSys> ssys;       // host copy (b, x filled per run)
+    std::vector<CgSmallGroup> groups;
+    SmallCtl ctl;                       // host copy of the control words
+    int64_t sbricks;                    // bricks of the largest group
+    CgSmallSys* d_ssys;
+    CgSmallGroup* d_groups;
+    SmallCtl* d_ctl;
+    int32_t h_err;
+    std::vector<int64_t> rows, len;   // unknowns of each system, values of its r, p and q
+    void* arena;               // r, p, q, partials, scalars and tables of all systems
     CgScalars* d_S;
     CgScalars* h_S;            // host mirror of the scalars, n entries
 };
@@ -250,11 +270,109 @@ int cg_batch_destroy(hs_cg_batch_t b)
     int rc = HS_OK;
     cudaError_t e = cudaStreamSynchronize(b->stream);
     if (e != cudaSuccess) rc = cuda_fail(e, "cg_batch_destroy: synchronize");
-    dev_free(b->d_sys, b->stream);
     dev_free(b->arena, b->stream);
     delete[] b->h_S;
     delete b;
     return rc;
+}
+
+// Lays out a new batch and allocates its device memory.
+static int cg_batch_fill(hs_cg_batch* b, const hs_op* ops, int32_t n)
+{
+    b->rows.resize((size_t)n);
+    int64_t vec_total = 0, part_total = 0;
+    int64_t blocks = 0;
+    for (int32_t i = 0; i < n; ++i) {
+        const OpDev A = to_dev(&ops[i]);
+        b->rows[(size_t)i] = A.n;
+        b->len.push_back((cg_vector_len(A) + 1) & ~(int64_t)1);   // every vector starts 16-byte aligned
+        vec_total += b->len.back();
+        CgSmallSys ss;
+        memset(&ss, 0, sizeof(ss));
+        if (cg_small_shape(A, &ss)) {
+            b->small.push_back(i);
+            part_total += 2 * (int64_t)ss.bricks;
+            continue;
+        }
+        SysDev s;
+        memset(&s, 0, sizeof(s));
+        s.A = A;
+        s.nblocks = grid_for(s.A.n);
+        s.mode = spmv_mode(s.A, s.nblocks);
+        s.nshares = s.mode == SP_STAGED ? spmv_shares(s.nblocks) : s.nblocks;
+        b->has_mode[s.mode] = true;
+        s.block0 = (int32_t)blocks;
+        blocks += s.nblocks;
+        part_total += 2 * (int64_t)s.nblocks;
+        b->big.push_back(i);
+        b->sys.push_back(s);
+    }
+    if (blocks > INT32_MAX) {
+        return fail(HS_EINVAL, "cg_batch_create: batch too large");
+    }
+    b->total_blocks = (int32_t)blocks;
+    // Small systems that advance in step share a group, at most kCgSmallSystems
+    // (groups of fewer unknowns, whose vectors would stay in L2, measured slower:
+    // 64 systems of 22.9 M unknowns 149 ms in one group, 165 in groups of 6 M, 179
+    // of 3 M -- the phases' fixed costs weigh more), those with about equally many
+    // iterations ahead together: the count grows with 1 / sum_d 1/n_d^2.
+    auto difficulty = [&](int32_t i) {
+        const double x = ops[i].nx, y = ops[i].ny, z = ops[i].nz;
+        return 1.0 / (1.0 / (x * x) + 1.0 / (y * y) + 1.0 / (z * z));
+    };
+    std::stable_sort(b->small.begin(), b->small.end(),
+                     [&](int32_t p, int32_t q) { return difficulty(p) > difficulty(q); });
+    int64_t bricks = 0;
+    for (size_t k = 0; k < b->small.size(); ++k) {
+        if (k % kCgSmallSystems == 0) {
+            b->groups.push_back(CgSmallGroup{(int32_t)k, 0});
+            bricks = 0;
+        }
+        CgSmallSys ss;
+        memset(&ss, 0, sizeof(ss));
+        (void)cg_small_shape(to_dev(&ops[b->small[k]]), &ss);
+        b->ssys.push_back(ss);
+        b->groups.back().count += 1;
+        bricks += ss.bricks;
+        b->sbricks = std::max(b->sbricks, bricks);
+    }
+    auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
+    const size_t s_vec = align(sizeof(double) * 3 * (size_t)vec_total), s_part = align(sizeof(double) * (size_t)part_total);
+    const size_t s_S = align(sizeof(CgScalars) * (size_t)n), s_sys = align(sizeof(SysDev) * b->sys.size());
+    const size_t s_ssys = align(sizeof(CgSmallSys) * b->ssys.size());
+    const size_t s_groups = align(sizeof(CgSmallGroup) * b->groups.size());
+    const size_t bytes = s_vec + s_part + s_S + s_sys + s_ssys + s_groups + sizeof(SmallCtl);
+    cudaError_t e = dev_alloc(&b->arena, bytes, b->stream);
+    if (e != cudaSuccess) b->arena = nullptr;
+    if (e == cudaSuccess) {
+        b->h_S = new (std::nothrow) CgScalars[(size_t)n]();
+        if (!b->h_S) e = cudaErrorMemoryAllocation;
+    }
+    if (e != cudaSuccess) return cuda_fail(e, "cg_batch_create: allocation");
+    char* base = (char*)b->arena;
+    double* vec = (double*)base;
+    double* part = (double*)(base + s_vec);
+    b->d_S = (CgScalars*)(base + s_vec + s_part);
+    b->d_sys = (SysDev*)(base + s_vec + s_part + s_S);
+    b->d_ssys = (CgSmallSys*)(base + s_vec + s_part + s_S + s_sys);
+    b->d_groups = (CgSmallGroup*)(base + s_vec + s_part + s_S + s_sys + s_ssys);
+    b->d_ctl = (SmallCtl*)(base + s_vec + s_part + s_S + s_sys + s_ssys + s_groups);
+    auto take = [&](auto& s, int32_t i, int64_t partials) {
+        const int64_t len = b->len[(size_t)i];
+        s.r = vec;
+        s.p = vec + len;
+        s.q = vec + 2 * len;
+        vec += 3 * len;
+        s.S = b->d_S + i;
+        double* const p0 = part;
+        part += partials;
+        return p0;
+    };
+    for (size_t k = 0; k < b->sys.size(); ++k)
+        b->sys[k].partials = take(b->sys[k], b->big[k], 2 * (int64_t)b->sys[k].nblocks);
+    for (size_t k = 0; k < b->ssys.size(); ++k)
+        b->ssys[k].part = take(b->ssys[k], b->small[k], 2 * (int64_t)b->ssys[k].bricks);
+    return HS_OK;
 }
 
 int cg_batch_create(hs_cg_batch_t* out, const hs_op* ops, int32_t n, void* stream)
@@ -271,54 +389,15 @@ int cg_batch_create(hs_cg_batch_t* out, const hs_op* ops, int32_t n, void* strea
     if (!b) return fail(HS_ENOMEM, "cg_batch_create: host allocation failed");
     b->stream = (cudaStream_t)stream;
     b->n = n;
-    b->sys.resize((size_t)n);
-    b->rows.resize((size_t)n);
-    int64_t vec_total = 0, part_total = 0;
-    int64_t blocks = 0;
-    for (int32_t i = 0; i < n; ++i) {
-        SysDev& s = b->sys[(size_t)i];
-        memset(&s, 0, sizeof(s));
-        s.A = to_dev(&ops[i]);
-        s.nblocks = grid_for(s.A.n);
-        s.mode = spmv_mode(s.A, s.nblocks);
-        s.nshares = s.mode == SP_STAGED ? spmv_shares(s.nblocks) : s.nblocks;
-        b->has_mode[s.mode] = true;
-        s.block0 = (int32_t)blocks;
-        blocks += s.nblocks;
-        b->rows[(size_t)i] = s.A.n;
-        vec_total += (s.A.n + 1) & ~(int64_t)1;   // every vector starts 16-byte aligned
-        part_total += 2 * (int64_t)s.nblocks;
+    int rc = HS_OK;
+    try {
+        rc = cg_batch_fill(b, ops, n);
+    } catch (const std::bad_alloc&) {
+        rc = fail(HS_ENOMEM, "cg_batch_create: host allocation failed");
     }
-    if (blocks > INT32_MAX) {
-        delete b;
-        return fail(HS_EINVAL, "cg_batch_create: batch too large");
-    }
-    b->total_blocks = (int32_t)blocks;
-    const size_t bytes = sizeof(double) * (size_t)(3 * vec_total + part_total) + sizeof(CgScalars) * (size_t)n;
-    cudaError_t e = dev_alloc(&b->arena, bytes, b->stream);
-    if (e == cudaSuccess) e = dev_alloc((void**)&b->d_sys, sizeof(SysDev) * (size_t)n, b->stream);
-    if (e == cudaSuccess) {
-        b->h_S = new (std::nothrow) CgScalars[(size_t)n]();
-        if (!b->h_S) e = cudaErrorMemoryAllocation;
-    }
-    if (e != cudaSuccess) {
-        const int rc = cuda_fail(e, "cg_batch_create: allocation");
+    if (rc != HS_OK) {
         cg_batch_destroy(b);
         return rc;
-    }
-    double* base = (double*)b->arena;
-    double* part = base + 3 * vec_total;
-    b->d_S = (CgScalars*)(part + part_total);
-    int64_t off = 0, poff = 0;
-    for (int32_t i = 0; i < n; ++i) {
-        SysDev& s = b->sys[(size_t)i];
-        s.r = base + off;
-        s.p = base + vec_total + off;
-        s.q = base + 2 * vec_total + off;
-        s.partials = part + poff;
-        s.S = b->d_S + i;
-        off += (s.A.n + 1) & ~(int64_t)1;
-        poff += 2 * (int64_t)s.nblocks;
     }
     *out = b;
     return HS_OK;
@@ -331,15 +410,32 @@ int cg_batch_run(hs_cg_batch_t b, const void* const* bs, void* const* xs, double
     if (!(rtol >= 0.0) || !std::isfinite(rtol)) return fail(HS_EINVAL, "cg_batch_run: bad rtol");
     if (max_iter < 0) return fail(HS_EINVAL, "cg_batch_run: max_iter < 0");
     const int n = b->n;
-    for (int i = 0; i < n; ++i) {
+    for (int i = 0; i < n; ++i)
         if (!bs[i] || !xs[i]) return fail(HS_EINVAL, "cg_batch_run: NULL vector of system %d", i);
-        b->sys[(size_t)i].b = (const double*)bs[i];
-        b->sys[(size_t)i].x = (double*)xs[i];
-        b->sys[(size_t)i].max_iter = max_iter;
+    for (size_t k = 0; k < b->sys.size(); ++k) {
+        b->sys[k].b = (const double*)bs[b->big[k]];
+        b->sys[k].x = (double*)xs[b->big[k]];
+        b->sys[k].max_iter = max_iter;
     }
-    HS_TRY_CUDA(cudaMemcpyAsync(b->d_sys, b->sys.data(), sizeof(SysDev) * (size_t)n, cudaMemcpyHostToDevice,
-                                b->stream),
-                "cg_batch_run: system table");
+    for (size_t k = 0; k < b->ssys.size(); ++k) {
+        b->ssys[k].b = (const double*)bs[b->small[k]];
+        b->ssys[k].x = (double*)xs[b->small[k]];
+        b->ssys[k].max_iter = max_iter;
+    }
+    if (!b->sys.empty())
+        HS_TRY_CUDA(cudaMemcpyAsync(b->d_sys, b->sys.data(), sizeof(SysDev) * b->sys.size(), cudaMemcpyHostToDevice,
+                                    b->stream),
+                    "cg_batch_run: system table");
+    if (!b->ssys.empty()) {
+        HS_TRY_CUDA(cudaMemcpyAsync(b->d_ssys, b->ssys.data(), sizeof(CgSmallSys) * b->ssys.size(),
+                                    cudaMemcpyHostToDevice, b->stream),
+                    "cg_batch_run: system table");
+        HS_TRY_CUDA(cudaMemcpyAsync(b->d_groups, b->groups.data(), sizeof(CgSmallGroup) * b->groups.size(),
+                                    cudaMemcpyHostToDevice, b->stream),
+                    "cg_batch_run: group table");
+        HS_TRY_CUDA(cudaMemcpyAsync(b->d_ctl, &b->ctl, sizeof(SmallCtl), cudaMemcpyHostToDevice, b->stream),
+                    "cg_batch_run: control words");
+    }
     for (int i = 0; i < n; ++i) {
         memset(&b->h_S[i], 0, sizeof(CgScalars));
         b->h_S[i].rtol = rtol;
@@ -350,18 +446,26 @@ int cg_batch_run(hs_cg_batch_t b, const void* const* bs, void* const* xs, double
     const int G = b->total_blocks;
 #define CGB_LAUNCH(kern, what)                                                 \
     do {                                                                       \
-        kern<<<G, kCgBlock, 0, b->stream>>>(b->d_sys, n);                      \
+        kern<<<G, kCgBlock, 0, b->stream>>>(b->d_sys, nbig);                      \
         HS_CHECK_LAUNCH(what);                                                 \
     } while (0)
     // the iteration kernels launch as dependent launches: each waits on entry
     // for the kernel before it, and its launch overlaps that kernel's tail
 #define CGB_LAUNCH_DEP(kern, what)                                                             \
     do {                                                                                       \
-        HS_TRY_CUDA(launch_dependent(kern, G, kCgBlock, b->stream, b->d_sys, n), "cg batch: kernel launch"); \
+        HS_TRY_CUDA(launch_dependent(kern, G, kCgBlock, b->stream, b->d_sys, nbig), "cg batch: kernel launch"); \
         HS_CHECK_LAUNCH(what);                                                                 \
     } while (0)
-    CGB_LAUNCH(k_cgb_apply_x, "cg batch: A x0 kernel");
-    CGB_LAUNCH(k_cgb_start, "cg batch: start kernel");
+    if (!b->ssys.empty()) {
+        const int rc_ = cg_small_launch(b->d_ssys, b->d_groups, (int)b->groups.size(), b->ssys.size() == 1, b->sbricks,
+                                        b->d_ctl->bar, &b->d_ctl->err, b->stream);
+        if (rc_ != HS_OK) return rc_;
+    }
+    const int nbig = (int)b->sys.size();
+    if (nbig) {
+        CGB_LAUNCH(k_cgb_apply_x, "cg batch: A x0 kernel");
+        CGB_LAUNCH(k_cgb_start, "cg batch: start kernel");
+    }
     int32_t enqueued = 0;
     int chunk = 4;
     for (;;) {
@@ -370,14 +474,14 @@ int cg_batch_run(hs_cg_batch_t b, const void* const* bs, void* const* xs, double
                     "cg_batch_run: scalar readback");
         HS_TRY_CUDA(cudaStreamSynchronize(b->stream), "cg_batch_run: synchronize");
         bool all = true;
-        for (int i = 0; i < n; ++i)
+        for (int32_t i : b->big)
             if (!b->h_S[i].done && b->h_S[i].iters < max_iter) all = false;
         if (all || enqueued >= max_iter) break;
         const int32_t todo = (max_iter - enqueued < chunk) ? max_iter - enqueued : chunk;
         for (int32_t t = 0; t < todo; ++t) {
             if (b->has_mode[SP_STAGED]) {
                 HS_TRY_CUDA(launch_dependent(k_cgb_spmv_dot<SP_STAGED, kSpBlock, kSpMinBlocks>, G, kSpBlock, b->stream, b->d_sys,
-                                             n),
+                                             nbig),
                             "cg batch: kernel launch");
                 HS_CHECK_LAUNCH("cg batch: spmv+dot kernel");
             }
@@ -390,18 +494,25 @@ int cg_batch_run(hs_cg_batch_t b, const void* const* bs, void* const* xs, double
         if (chunk < 32) chunk *= 2;
     }
     // zero right-hand sides have the solution 0
-    for (int i = 0; i < n; ++i)
+    for (int32_t i : b->big)
         if (b->h_S[i].zero_rhs)
             HS_TRY_CUDA(cudaMemsetAsync(xs[i], 0, sizeof(double) * (size_t)b->rows[(size_t)i], b->stream),
                         "cg_batch_run: zero solution");
-    CGB_LAUNCH(k_cgb_apply_x, "cg batch: A x kernel");
-    CGB_LAUNCH(k_cgb_resid, "cg batch: residual kernel");
+    if (nbig) {
+        CGB_LAUNCH(k_cgb_apply_x, "cg batch: A x kernel");
+        CGB_LAUNCH(k_cgb_resid, "cg batch: residual kernel");
+    }
 #undef CGB_LAUNCH
 #undef CGB_LAUNCH_DEP
     HS_TRY_CUDA(cudaMemcpyAsync(b->h_S, b->d_S, sizeof(CgScalars) * (size_t)n, cudaMemcpyDeviceToHost,
                                 b->stream),
                 "cg_batch_run: scalar readback");
+    b->h_err = 0;
+    if (!b->ssys.empty())
+        HS_TRY_CUDA(cudaMemcpyAsync(&b->h_err, &b->d_ctl->err, sizeof(int32_t), cudaMemcpyDeviceToHost, b->stream),
+                    "cg_batch_run: control words");
     HS_TRY_CUDA(cudaStreamSynchronize(b->stream), "cg_batch_run: synchronize");
+    if (b->h_err) return fail(HS_ETIMEOUT, "cg_batch_run: a bounded wait in the small-system kernel ran out");
     int rc = HS_OK;
     for (int i = 0; i < n; ++i) {
         const CgScalars& f = b->h_S[i];

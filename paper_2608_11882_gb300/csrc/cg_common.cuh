@@ -30,6 +30,7 @@ struct CgScalars {
     // operator): the kernel that forms p_i folds its values in and clears slot
     // (i+1) % 3; the SpMV of iteration i reads slot i % 3.
     unsigned long long pmax[3];
+    double rho2[2];    // cg_small.cu: r.r of iteration i in slot i % 2
 };
 
 constexpr int kCgBlock = 256;
@@ -506,6 +507,8 @@ int spmv_tma_launch(const CUtensorMap& map, const OpDev& A, double* q, double* p
 int check_op(const hs_op* A);
 OpDev to_dev(const hs_op* A);
 int grid_for(int64_t n);
+size_t cg_partials(const OpDev& A, int grid);
+int cg_create_vectors(hs_cg_t* out, const hs_op* A, void* stream, bool need_p);
 int launch_apply(const OpDev& A, const double* p, double* y, cudaStream_t s);
 
 }  // namespace hcg
@@ -517,7 +520,9 @@ struct hs_cg {
     double* r;
     double* p;
     double* q;
-    double* partials;      // 2 * grid doubles
+    void* arena;           // device allocation behind ctl, S, partials, r, p and q; null: the caller's scratch
+    char* ctl;             // control words of the small-system kernel (cg_small.cuh), S among them
+    double* partials;      // cg_partials(A, grid) doubles
     hcg::CgScalars* S;     // device scalars
     hcg::CgScalars* S_host;  // host mirror of the scalars
     void* owned[3];        // device copies of host CSR arrays

@@ -743,7 +743,7 @@ int cg_create_mixed(hs_cg_t* out, const hs_op* A, const hs_cg_mixed_opts* opts, 
         return fail(HS_EINVAL, "cg_create_mixed: inner_rtol %g not in (0, 1)", inner_rtol);
     if (max_inner < 1) return fail(HS_EINVAL, "cg_create_mixed: max_inner < 1");
     hs_cg_t c = nullptr;
-    int rc = cg_create(&c, A, stream);
+    int rc = cg_create_vectors(&c, A, stream, false);   // no FP64 direction
     if (rc != HS_OK) return rc;
     CgMixed* m = new (std::nothrow) CgMixed();
     if (!m) {
@@ -759,11 +759,9 @@ int cg_create_mixed(hs_cg_t* out, const hs_op* A, const hs_cg_mixed_opts* opts, 
     const cudaStream_t s = c->stream;
     for (float** v : {&m->d, &m->r, &m->p, &m->q})
         if (e == cudaSuccess) e = dev_alloc((void**)v, sizeof(float) * (size_t)n, s);
-    // the FP64 residual and A x live in the context's FP64 r and q; its p is not needed
+    // the FP64 residual and A x live in the context's FP64 r and q
     m->r64 = c->r;
     m->q64 = c->q;
-    dev_free(c->p, s);
-    c->p = nullptr;
     if (e == cudaSuccess) e = dev_alloc((void**)&m->partials, sizeof(double) * 3 * (size_t)G, s);
     if (e == cudaSuccess) e = dev_alloc((void**)&m->S, sizeof(MxScalars), s);
     if (e == cudaSuccess) {

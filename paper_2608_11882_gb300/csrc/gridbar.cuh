@@ -1,5 +1,5 @@
-// Grid-wide barrier between the co-resident blocks of one cooperative launch,
-// carrying the largest of the blocks' values.
+// Barrier between the blocks of one cooperative launch, carrying the largest of
+// the blocks' values.
 //
 // One 64-bit word per phase counts the arrivals, so a block arrives with a
 // single reduction (no value comes back) and one of its threads polls one
@@ -9,8 +9,7 @@
 // when some block still holds the previous value and none exceeds it, the
 // arrival word alone gives the result.  Blocks with another value also fold it
 // into a second word, which is read only when the first does not decide.
-// Three sets of words are used in turn; block 0 clears the set after next's
-// before it arrives, when every block has left it.  (All blocks reading all
+// Three sets of words are used in turn; block 0 clears the next set before it arrives, when every block has left it.  (All blocks reading all
 // blocks' values instead of counting measured 3.6 us more per phase at 128
 // blocks.)
 //
@@ -63,8 +62,8 @@ __device__ __forceinline__ void grid_arrive(unsigned long long* bar, int ph, uns
 // largest value.  False when the wait ran out or another block gave up.
 __device__ __forceinline__ bool grid_wait(unsigned long long* bar, int ph, unsigned prev, unsigned* m, int* err)
 {
+    const unsigned need = gridDim.x;
     unsigned long long* ctr = bar + (ph % 3) * kGridBarStride;
-    const unsigned long long need = gridDim.x;
     unsigned long long v = ld_acquire_u64(ctr);
     if ((v & 0xfffffull) != need) {
         const long long t0 = clock64();
