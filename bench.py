@@ -69,9 +69,7 @@ HEAT_MODES = {
 # Algorithmic bytes of the other rows (read each input once, write each output once):
 #  * batched heat: 16 B per lattice-point update of an FP64 grid, 8 B of an FP32 grid;
 #  * the paper's variable-coefficient update: u, kappa and dt f read, u' written --
-#    32 B (FP64) / 16 B (FP32) per update; the FP64 form is bound by the FP64 pipe
-#    at 23 operations per update (per axis 4 additions, a multiply and an FMA for
-#    the face differences; 5 to add dt f and the three scaled differences);
+#    32 B (FP64) / 16 B (FP32) per update;
 #  * CG per unknown and iteration: SpMV 16 B (read p, write q), x/r update 48 B
 #    (read x, p, r, q; write x, r), p update 24 B (read r, p; write p) = 88 B
 #    matrix-free; CSR adds 12 B per stored entry and 4 B of row pointer per row;
@@ -81,7 +79,7 @@ HEAT_MODES = {
 #    p update 12 B; per refinement:
 #    FP64 SpMV 16 B (+ 12 B per entry, 4 B per row for CSR), residual 36 B
 #    (read b, A x; write r in FP64 and r, p, d in FP32), correction 20 B.
-VK_FP64_OPS_PER_LUP = 2    # FP64 variable-kappa update, exact-sum form: u + dt f, then one FMA
+VK_FP64_OPS_PER_LUP = 2.5  # FP64 variable-kappa update, exact-sum form: u + dt f, one FMA, half a conversion
 CG_BYTES_PER_ROW = 88
 MIXED_INNER_BYTES_PER_ROW = {"matrix_free": 40, "csr": 44}
 MIXED_REFINE_BYTES_PER_ROW = 72
@@ -269,15 +267,12 @@ def paper_problem_side(pkg, stream, hbm_gbs, peak_kind, n=510, steps=500):
             ms = e0.elapsed_time(e1)
         lups = float(n) ** 3 * steps
         out[dtype] = {"glups": lups / (ms * 1e-3) / 1e9, "ms": ms}
-        # FP64: u read and written, three face-sum arrays of kappa, dt f (48 B);
-        # FP32: u read and written, kappa, dt f (16 B).  The cubic FP64 grid
-        # runs the exact-sum form (2 FP64 instructions per update, the operator
-        # sum in 128-bit integers), bound by integer issue and load latency:
-        # its roofline object is HBM at 48 B per update, with the FP64 pipe's
-        # share beside it
-        bpl = 48 if dtype == "f64" else 16
-        kname = "k_vk_interior_xs + k_vk_boundary_xs (exact sum)" if dtype == "f64" else \
-            "k_vk_interior_f4 + k_vk_boundary<float>"
+        # u read and written, kappa and dt f read: 32 B (FP64), 16 B (FP32).  FP64
+        # runs the exact-sum form (fluxes in integers, 2.5 FP64 instructions per
+        # update), bound by instruction issue: its roofline object is HBM at 32 B
+        # per update, with the FP64 pipe's share beside it
+        bpl = 32 if dtype == "f64" else 16
+        kname = "k_vk_xs (exact sum)" if dtype == "f64" else "k_vk_f4"
         hbm = hbm_roofline(kname, lups * bpl, ms, hbm_gbs, peak_kind, bytes_per_lup=bpl)
         if dtype == "f64":
             rate = lups * VK_FP64_OPS_PER_LUP / (ms * 1e-3) / 1e12

@@ -86,15 +86,13 @@ extern "C" {
  * (the paper does not print D; this is the reading consistent with its
  * beta = dt/(2h^2)).  Here r means dt / h_min^2 (the paper's choice is
  * dt = h^2/(12 kappa_max), r = 1/(12 * 0.95)); the stability bound is
- * r <= 1/(6 kappa_max).  The coefficients (on every node, boundary included)
- * and dt f live on the device beside u, as in the paper's 1-GPU Baseline:
- * kappa itself for HS_F32, for HS_F64 the three face sums k[i+1] + k[i] of
- * each node (constant in time; the same values the formula forms).  For
- * HS_F64 the operator sums are formed exactly in integers on the field's
+ * r <= 1/(6 kappa_max).  kappa (on every node, boundary included) and dt f live
+ * on the device beside u, as in the paper's 1-GPU Baseline.  For HS_F64 each
+ * face's flux (kappa + kappa_nb)(u_nb - u) is formed in integers on the field's
  * fixed-point scale (its largest exponent, tracked on the device as for the
- * default FP64 arithmetic) and rounded once -- the whole sum on a cubic grid,
- * each axis's sum otherwise: error below 6 * 2 * 1.9 * 4 * 2^-57 max|u| beta
- * plus a few roundings per step; fields outside [2^-903, 2^1007] in magnitude
+ * default FP64 arithmetic), the six are summed exactly and rounded once: error
+ * below 30 * 2^-57 max|u| beta plus a few roundings per step; fields outside
+ * [2^-903, 2^1007] in magnitude
  * step in FP64 arithmetic.  HS_F64 or
  * HS_F32; excludes HS_FIXED64, HS_EXACT_ROUNDING, HS_SCHED_FULL and tdepth > 1;
  * cannot join a heat batch. */
@@ -158,9 +156,7 @@ int heat_buffer_bytes(const hs_heat_desc* desc, size_t* bytes);
 
 /* Device bytes heat_create would allocate for desc (for admission control):
  * the two field buffers unless the caller supplies them, and the per-step
- * state of the exact-sum and FIXED64 arithmetics (and the coefficient
- * arrays and dt f for HS_VARKAPPA: two fields' worth for HS_F32, four for
- * HS_F64). */
+ * state of the exact-sum and FIXED64 arithmetics (and kappa and dt f for HS_VARKAPPA, two fields' worth). */
 int heat_device_bytes(const hs_heat_desc* desc, size_t* bytes);
 
 /* Load the interior field u (nx*ny*nz elements of the handle's dtype, x

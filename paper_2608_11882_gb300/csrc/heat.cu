@@ -313,9 +313,11 @@ struct hs_heat {
     uint32_t tbox[2];      // box of maps[]
     uint32_t sbox[2];      // box of smaps[]
     int kc_stream;         // k-planes per block of the streaming Interior kernel
-    void* kap;             // HS_VARKAPPA: FP32 kappa on every padded node, FP64 its three face sums
+    void* kap;             // HS_VARKAPPA: kappa on every padded node
     void* fdt;             // HS_VARKAPPA: dt f on the interior
     double vbx, vby, vbz;  // HS_VARKAPPA: dt / (2 h_d^2)
+    int kappa_ok;          // HS_VARKAPPA, FP64: kappa allows the exact-sum form
+    CUtensorMap vmaps[4];  // HS_VARKAPPA, FP64: TMA maps of the two buffers, kappa and dt f
     // Large grids run each step's Boundary kernel on a side stream, beside the
     // Interior kernel: forked from `stream` after the previous step (ev_fork)
     // and joined back before the next one (ev_join).  Null: one stream.
@@ -422,9 +424,14 @@ int pick_kchunk(const HeatGeom& g, uint32_t flags = 0, int dtype = HS_F64)
     // blocks in flight) measured 340 GLUP/s at 8 planes against 265 at the
     // 102 planes of the rule below (510^3)
     if ((flags & HS_VARKAPPA) && dtype == HS_F32) return g.nz > 2 ? std::min(8, g.nz - 2) : 1;
-    // the FP64 variable-kappa kernels: 32-plane chunks (77.0 GLUP/s at 510^3
-    // against 75.8 with the 102 of the rule below)
-    if (flags & HS_VARKAPPA) return g.nz > 2 ? std::min(32, g.nz - 2) : 1;
+    // the FP64 variable-kappa kernel: about eight waves of three blocks per SM, in
+    // chunks of 4 to 64 planes (510^3: 64 planes 140 GLUP/s, 32 139, 16 135, 128
+    // 135; 96^3: 4 planes 16.5 us per step, 16 20.7, 32 35)
+    if (flags & HS_VARKAPPA) {
+        const int64_t tiles = (int64_t)((g.nx + 63) / 64) * ((g.ny + 7) / 8);
+        const int64_t kc = (tiles * g.nz + kNumSMs * 24 - 1) / (kNumSMs * 24);
+        return (int)std::min<int64_t>(std::max<int64_t>(4, std::min<int64_t>(kc, 64)), g.nz);
+    }
     const int64_t blocks_xy = (int64_t)((g.nx + kBX - 1) / kBX) * ((g.ny + kBY - 1) / kBY);
     const int64_t target = (int64_t)kNumSMs * 8 * 4;   // about four waves of 8 blocks per SM
     const int64_t nzi = g.nz > 2 ? g.nz - 2 : 1;
@@ -535,10 +542,12 @@ int launch_part(hs_heat* h, Part p, T param, cudaStream_t s)
     return launch_full_t<T, EXACT>(h, param);
 }
 
-int vk_part(hs_heat* h, Part p, cudaStream_t s)
+// Planes [kbeg, kend) of a step of the variable-coefficient problem.
+int vk_planes(hs_heat* h, int kbeg, int kend, cudaStream_t s)
 {
-    VkCall c;
-    c.part = (p == P_INTERIOR) ? 0 : 1;
+    VkCall c = {};
+    c.kbeg = kbeg;
+    c.kend = kend;
     c.f64 = h->dtype == HS_F64;
     c.src = h->buf[h->cur];
     c.dst = h->buf[1 - h->cur];
@@ -552,7 +561,21 @@ int vk_part(hs_heat* h, Part p, cudaStream_t s)
     c.stream = s;
     c.fx = h->fx;   // FP64 only
     c.m3 = (int)(h->fxseq % 3);
+    c.err = h->err;
+    c.umap = &h->vmaps[h->cur];
+    c.kmap = &h->vmaps[2];
+    c.fmap = &h->vmaps[3];
+    c.exact = h->kappa_ok;
     return vk_launch(c);
+}
+
+int vk_part(hs_heat* h, Part p, cudaStream_t s)
+{
+    const int nz = h->g.nz;
+    if (p == P_FULL) return vk_planes(h, 0, nz, s);
+    if (p == P_INTERIOR) return vk_planes(h, 1, nz - 1, s);
+    const int rc = vk_planes(h, 0, 1, s);
+    return rc != HS_OK || nz < 2 ? rc : vk_planes(h, nz - 1, nz, s);
 }
 
 // Launches one part of a step.  The Boundary kernel goes to stream s (the
@@ -835,9 +858,8 @@ int heat_device_bytes(const hs_heat_desc* desc, size_t* bytes)
     *bytes = user_bufs ? 0 : 2 * (size_t)g.total * elem_size(desc->dtype);
     const Arith a = pick_arith(desc);
     if (a == A_FX64 || a == A_F64_XS) *bytes += sizeof(FxState);
-    if (desc->flags & HS_VARKAPPA)   // coefficients (FP64: three face arrays) and dt f
-        *bytes += (desc->dtype == HS_F64 ? 4 : 2) * (size_t)g.total * elem_size(desc->dtype) +
-                  (desc->dtype == HS_F64 ? sizeof(FxState) : 0);
+    if (desc->flags & HS_VARKAPPA)   // kappa and dt f
+        *bytes += 2 * (size_t)g.total * elem_size(desc->dtype) + (desc->dtype == HS_F64 ? sizeof(FxState) : 0);
     return HS_OK;
 }
 
@@ -938,11 +960,9 @@ int heat_create(hs_heat_t* out, const hs_heat_desc* desc)
     if (h->arith == A_FX64 || h->arith == A_F64_XS) h->fx = fx_state;
     if (h->flags & HS_VARKAPPA) {
         const size_t bytes = (size_t)h->g.total * h->elem;
-        // FP64 keeps the three face sums of kappa, FP32 kappa itself
-        const size_t cbytes = h->dtype == HS_F64 ? 3 * bytes : bytes;
-        cudaError_t e = dev_alloc(&h->kap, cbytes, h->stream);
+        cudaError_t e = dev_alloc(&h->kap, bytes, h->stream);
         if (e == cudaSuccess) e = dev_alloc(&h->fdt, bytes, h->stream);
-        if (e == cudaSuccess) e = cudaMemsetAsync(h->kap, 0, cbytes, h->stream);
+        if (e == cudaSuccess) e = cudaMemsetAsync(h->kap, 0, bytes, h->stream);
         if (e == cudaSuccess) e = cudaMemsetAsync(h->fdt, 0, bytes, h->stream);
         if (e != cudaSuccess) {
             rc = cuda_fail(e, "heat_create: kappa/source arrays");
@@ -961,35 +981,42 @@ int heat_create(hs_heat_t* out, const hs_heat_desc* desc)
         c.fdt = h->fdt;
         c.g = &h->g;
         c.stream = h->stream;
-        int face_off = 1;
+        int kappa_off = 1;
         if (c.f64) {
-            e = dev_alloc((void**)&c.face_off, sizeof(int), h->stream);
-            if (e == cudaSuccess) e = cudaMemsetAsync(c.face_off, 0, sizeof(int), h->stream);
+            e = dev_alloc((void**)&c.kappa_off, sizeof(int), h->stream);
+            if (e == cudaSuccess) e = cudaMemsetAsync(c.kappa_off, 0, sizeof(int), h->stream);
             if (e != cudaSuccess) {
-                rc = cuda_fail(e, "heat_create: face-sum check word");
+                rc = cuda_fail(e, "heat_create: kappa check word");
                 heat_destroy(h);
                 return rc;
             }
         }
         rc = vk_init(c, dt);
         if (rc == HS_OK && c.f64) {
-            cudaError_t e2 = cudaMemcpyAsync(&face_off, c.face_off, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
+            cudaError_t e2 = cudaMemcpyAsync(&kappa_off, c.kappa_off, sizeof(int), cudaMemcpyDeviceToHost, h->stream);
             if (e2 == cudaSuccess) e2 = cudaStreamSynchronize(h->stream);
-            if (e2 != cudaSuccess) rc = cuda_fail(e2, "heat_create: face-sum check");
+            if (e2 != cudaSuccess) rc = cuda_fail(e2, "heat_create: kappa check");
         }
-        if (c.face_off) dev_free(c.face_off, h->stream);
+        if (c.kappa_off) dev_free(c.kappa_off, h->stream);
         if (rc != HS_OK) {
             heat_destroy(h);
             return rc;
         }
-        // FP64 with every face sum of kappa in [1, 2): the exact-sum form,
-        // which tracks the field's largest exponent step by step
-        if (h->dtype == HS_F64 && face_off == 0) h->fx = fx_state;
+        if (h->dtype == HS_F64) h->fx = fx_state;   // the exact-sum form tracks the field's largest exponent
+        h->kappa_ok = kappa_off == 0;
+        if (h->dtype == HS_F64) {
+            const int em = vk_maps(h->vmaps, h->buf, h->kap, h->fdt, h->g);
+            if (em != 0) {
+                rc = cuda_fail((cudaError_t)em, "heat_create: TMA tensor map (variable kappa)");
+                heat_destroy(h);
+                return rc;
+            }
+        }
     }
     // A Boundary kernel beside the Interior one pays for its extra API calls
     // once the Interior kernel takes tens of microseconds (2^22 points and up).
     const int64_t npts = (int64_t)h->g.nx * h->g.ny * h->g.nz;
-    if (!(h->flags & HS_SCHED_FULL) && h->tdepth == 1 && npts >= kForkMinPoints && h->g.nz >= 3) {
+    if (!(h->flags & (HS_SCHED_FULL | HS_VARKAPPA)) && h->tdepth == 1 && npts >= kForkMinPoints && h->g.nz >= 3) {
         cudaError_t e = cudaStreamCreateWithFlags(&h->bstream, cudaStreamNonBlocking);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_fork, cudaEventDisableTiming);
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&h->ev_join, cudaEventDisableTiming);
@@ -1095,8 +1122,8 @@ int heat_step(hs_heat_t h, int64_t n_steps)
     }
     for (int64_t m = 0; m < n_steps; ++m) {
         int rc;
-        if (h->flags & HS_SCHED_FULL) {
-            rc = do_part(h, P_FULL);
+        if ((h->flags & HS_SCHED_FULL) || ((h->flags & HS_VARKAPPA) && !h->timing)) {
+            rc = do_part(h, P_FULL);   // variable kappa: all planes in one launch
         } else if (h->bstream) {
             // Interior on the handle's stream, Boundary beside it on the side
             // stream (the two write disjoint planes of the new level and fold

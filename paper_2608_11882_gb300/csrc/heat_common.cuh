@@ -308,26 +308,29 @@ constexpr int kXsRowsPerThread = 2;
 constexpr int kXsStages = 4;
 inline int stream_rows_for(int arith) { return arith == A_F64_XS ? kXsRows : kStreamRowsHost; }
 
-// One launch of a variable-coefficient kernel (heat_vk.cu).
+// One launch of a variable-coefficient kernel (heat_vk.cu) over the planes
+// [kbeg, kend).
 struct VkCall {
-    int part;                // 0: Interior (planes 1..nz-2), 1: Boundary (planes 0, nz-1)
+    int kbeg, kend;
     int f64;                 // 1: FP64, 0: FP32
     const void* src;
     void* dst;
-    void* kap;               // FP32: kappa on every padded node; FP64: the three face
-                             // sums of kappa (x, y, z arrays of g.total elements each)
+    void* kap;               // kappa on every padded node
     void* fdt;               // dt f on the interior
     const HeatGeom* g;
     double bx, by, bz;       // dt / (2 h_d^2)
     int kchunk;
     cudaStream_t stream;
-    FxState* fx;             // FP64: the per-step maxima of the exact-sum form
-                             // (nullptr: the FP64 form, no maxima)
+    FxState* fx;             // FP64: the per-step maxima
     int m3;                  // slot of the current field in fx
-    int* face_off;           // vk_init, FP64: device word set to 1 if a face sum lies outside [1, 2)
+    int* err;                // device error word of the bounded waits
+    const CUtensorMap *umap, *kmap, *fmap;   // FP64: vk_maps of src, kappa and dt f
+    int exact;               // FP64: every kappa is in [0.5, 1), as the exact-sum form needs
+    int* kappa_off;          // vk_init, FP64: device word set to 1 if one is not
 };
 int vk_init(const VkCall& c, double dt);
 int vk_launch(const VkCall& c);
+int vk_maps(CUtensorMap (&maps)[4], void* const (&buf)[2], void* kap, void* fdt, const HeatGeom& g);
 
 // One launch of the multi-step kernel (heat_multi.cu): `steps` whole steps.
 struct MultiCall {

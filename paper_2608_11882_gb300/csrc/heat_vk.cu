@@ -8,29 +8,28 @@
 // coefficients and dt f are arrays resident beside u, dt f on the interior.
 // Interior and Boundary kernels as for the constant-coefficient update.
 //
-// FP32 keeps kappa on every node of the padded box (16 bytes per update:
-// the kernel is bound by HBM, where three face arrays would cost more than the
-// six additions they save).  FP64 keeps the three face sums k[i+1] + k[i] of
-// each node instead (constant in time, formed once at creation, bit for bit
-// the sums the formula forms every step), 48 bytes per update, and forms the
-// operator sums exactly in 128-bit integers on the field's fixed-point scale,
-// each rounded once: 2 FP64 instructions per update on a cubic grid (one beta
-// for every axis: the paper's case), 5 otherwise.  Fields outside the exact
-// form's exponent range use the FP64 form, 16 FP64 instructions per update
-// with the z difference u[k+1] - u[k] carried to the next plane (23 with kappa
-// itself).
+// Every node of the padded box keeps its kappa: u, kappa and dt f in, u' out, 32
+// bytes per FP64 update and 16 per FP32 update.  FP64 forms the operator sum in
+// integers on the field's fixed-point scale -- each face's flux kappa dU from
+// three 32-bit products, the six fluxes summed in 64 bits and rounded to a
+// double once -- and spends two or three FP64 instructions per update, where
+// the formula takes 23.  Fields outside that form's exponent range use the
+// formula itself.
 #include <cmath>
 
 #include "heat_common.cuh"
+#include "tma.cuh"
 
 namespace hcg {
 
 constexpr int kVkBX = 32, kVkBY = 8;
 
 // kappa on every padded node, dt f on interior nodes (zero on the boundary).
+// Sets *off = 1 if a kappa lies outside [0.5, 1), where xs_flux would not hold it
+// (0.5 + 0.45 s with s in [0, 1] never does).
 template <typename T>
 __global__ void __launch_bounds__(256) k_vk_init(T* __restrict__ kap, T* __restrict__ fdt, HeatGeom g,
-                                                 double dt)
+                                                 double dt, int* off)
 {
     const double hx = 1.0 / (g.nx + 1), hy = 1.0 / (g.ny + 1), hz = 1.0 / (g.nz + 1);
     const int64_t n = (int64_t)(g.nx + 2) * (g.ny + 2) * (g.nz + 2);
@@ -42,336 +41,12 @@ __global__ void __launch_bounds__(256) k_vk_init(T* __restrict__ kap, T* __restr
         const int K = (int)(jk / (g.ny + 2));
         const int64_t c = (int64_t)K * g.plane + (int64_t)J * g.pitch + g.lead - 1 + I;
         const double x = I * hx, y = J * hy, z = K * hz;
-        kap[c] = (T)(0.5 + 0.45 * sinpi(x) * sinpi(y) * sinpi(z));
+        const double k = 0.5 + 0.45 * sinpi(x) * sinpi(y) * sinpi(z);
+        kap[c] = (T)k;
+        if (off && !(k >= 0.5 && k < 1.0)) atomicOr(off, 1);
         const bool interior = I >= 1 && I <= g.nx && J >= 1 && J <= g.ny && K >= 1 && K <= g.nz;
         fdt[c] = interior ? (T)(dt * (1.0 + cospi(x) * cospi(y) * cospi(z))) : (T)0;
     }
-}
-
-// FP64: the three face sums of kappa on every padded node (f*[c] = kappa at the
-// node's +d neighbour + kappa at the node, zero where that neighbour lies
-// outside the padded box) and dt f on the interior.  The kappa values are the
-// same expression as k_vk_init's, so the sums are the bits the formula forms.
-// Sets *off = 1 if a face sum lies outside [1, 2), where the exact-sum form's
-// 53-bit significands would not hold it (kappa in [0.5, 1) keeps every face
-// sum inside).
-__global__ void __launch_bounds__(256) k_vk_init_faces(double* __restrict__ fc, double* __restrict__ fdt,
-                                                       HeatGeom g, double dt, int* off)
-{
-    const double hx = 1.0 / (g.nx + 1), hy = 1.0 / (g.ny + 1), hz = 1.0 / (g.nz + 1);
-    const int64_t n = (int64_t)(g.nx + 2) * (g.ny + 2) * (g.nz + 2);
-    auto kappa = [&](int I, int J, int K) {
-        return 0.5 + 0.45 * sinpi(I * hx) * sinpi(J * hy) * sinpi(K * hz);
-    };
-    for (int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; t < n;
-         t += (int64_t)gridDim.x * blockDim.x) {
-        const int I = (int)(t % (g.nx + 2));
-        const int64_t jk = t / (g.nx + 2);
-        const int J = (int)(jk % (g.ny + 2));
-        const int K = (int)(jk / (g.ny + 2));
-        const int64_t c = (int64_t)K * g.plane + (int64_t)J * g.pitch + g.lead - 1 + I;
-        const double kc = kappa(I, J, K);
-        const double sx = kappa(I + 1, J, K) + kc, sy = kappa(I, J + 1, K) + kc, sz = kappa(I, J, K + 1) + kc;
-        fc[c] = I <= g.nx ? sx : 0.0;
-        fc[g.total + c] = J <= g.ny ? sy : 0.0;
-        fc[2 * g.total + c] = K <= g.nz ? sz : 0.0;
-        auto out = [](double v) { return !(v >= 1.0 && v < 2.0); };
-        if ((I <= g.nx && out(sx)) || (J <= g.ny && out(sy)) || (K <= g.nz && out(sz))) atomicOr(off, 1);
-        const bool interior = I >= 1 && I <= g.nx && J >= 1 && J <= g.ny && K >= 1 && K <= g.nz;
-        fdt[c] = interior ? dt * (1.0 + cospi(I * hx) * cospi(J * hy) * cospi(K * hz)) : 0.0;
-    }
-}
-
-// One FP64 update from the face sums: cxp = k[i+1] + k[i], cxm = k[i] + k[i-1]
-// (the -x neighbour's +x face) and so on, and the z difference below the
-// point, dzm = u[k] - u[k-1], carried from the plane below.
-__device__ __forceinline__ double vk_point_faces(double uc, double uxm, double uxp, double uym, double uyp,
-                                                 double dzp, double dzm, double cxm, double cxp, double cym,
-                                                 double cyp, double czm, double czp, double f, double bx,
-                                                 double by, double bz)
-{
-    const double dx = __fma_rn(cxp, __dsub_rn(uxp, uc), -__dmul_rn(cxm, __dsub_rn(uc, uxm)));
-    const double dy = __fma_rn(cyp, __dsub_rn(uyp, uc), -__dmul_rn(cym, __dsub_rn(uc, uym)));
-    const double dz = __fma_rn(czp, dzp, -__dmul_rn(czm, dzm));
-    return __dadd_rn(__dadd_rn(uc, f), __fma_rn(bz, dz, __fma_rn(by, dy, __dmul_rn(bx, dx))));
-}
-
-__global__ void __launch_bounds__(kVkBX* kVkBY)
-    k_vk_interior_faces(const double* __restrict__ src, double* __restrict__ dst, const double* __restrict__ fc,
-                        const double* __restrict__ fdt, HeatGeom g, double bx, double by, double bz, int kbeg,
-                        int kend, int kchunk)
-{
-    const int i = blockIdx.x * kVkBX + threadIdx.x;
-    const int j = blockIdx.y * kVkBY + threadIdx.y;
-    if (i >= g.nx || j >= g.ny) return;
-    const int k0 = kbeg + (int)blockIdx.z * kchunk;
-    const int k1 = min(k0 + kchunk, kend);
-    if (k0 >= k1) return;
-    const int64_t P = g.plane, Y = g.pitch;
-    const double* fx = fc;
-    const double* fy = fc + g.total;
-    const double* fz = fc + 2 * g.total;
-    int64_t c = g.at(i, j, k0);
-    double uc = __ldg(src + c);
-    double dzm = __dsub_rn(uc, __ldg(src + c - P));
-    double czm = __ldg(fz + c - P);
-    for (int k = k0; k < k1; ++k) {
-        const double ua = __ldg(src + c + P), cza = __ldg(fz + c);
-        const double dzp = __dsub_rn(ua, uc);
-        dst[c] = vk_point_faces(uc, __ldg(src + c - 1), __ldg(src + c + 1), __ldg(src + c - Y),
-                                __ldg(src + c + Y), dzp, dzm, __ldg(fx + c - 1), __ldg(fx + c),
-                                __ldg(fy + c - Y), __ldg(fy + c), czm, cza, __ldg(fdt + c), bx, by, bz);
-        uc = ua;
-        dzm = dzp;
-        czm = cza;
-        c += P;
-    }
-}
-
-__global__ void __launch_bounds__(kVkBX* kVkBY)
-    k_vk_boundary_faces(const double* __restrict__ src, double* __restrict__ dst, const double* __restrict__ fc,
-                        const double* __restrict__ fdt, HeatGeom g, double bx, double by, double bz)
-{
-    const int i = blockIdx.x * kVkBX + threadIdx.x;
-    const int j = blockIdx.y * kVkBY + threadIdx.y;
-    if (i >= g.nx || j >= g.ny) return;
-    const int k = (blockIdx.z == 0) ? 0 : g.nz - 1;
-    const int64_t P = g.plane, Y = g.pitch;
-    const int64_t c = g.at(i, j, k);
-    const double* fx = fc;
-    const double* fy = fc + g.total;
-    const double* fz = fc + 2 * g.total;
-    const double uc = __ldg(src + c);
-    dst[c] = vk_point_faces(uc, __ldg(src + c - 1), __ldg(src + c + 1), __ldg(src + c - Y), __ldg(src + c + Y),
-                            __dsub_rn(__ldg(src + c + P), uc), __dsub_rn(uc, __ldg(src + c - P)),
-                            __ldg(fx + c - 1), __ldg(fx + c), __ldg(fy + c - Y), __ldg(fy + c),
-                            __ldg(fz + c - P), __ldg(fz + c), __ldg(fdt + c), bx, by, bz);
-}
-
-// ---- FP64, exact sum ------------------------------------------------------
-// The operator sums D_d = c_d+ (u_d+ - u) - c_d- (u - u_d-) on the field's
-// fixed-point scale: U the exact-sum integers of the u values (xsum.cuh, the
-// scale 2^(1080 - e) of the field's largest exponent field e, tracked per step
-// in the handle's FxState like the default FP64 arithmetic's), C the face
-// sums' 53-bit significands (every face sum of kappa = 0.5 + 0.45 s, s in
-// [0, 1], lies in [1, 2), so C = c 2^52 exactly; heat_create checks it), each
-// product C dU exact and their sums exact in 128 bits.  On a cubic grid (one
-// beta for every axis, the paper's case) the whole operator sum is rounded
-// once and u' = fma(beta, D, u + dt f): two FP64 instructions per update
-// instead of sixteen; otherwise each axis sum is rounded once and combined as
-// the FP64 form combines them, five FP64 instructions.  The error against the
-// same formula in exact arithmetic is below 6 * 2 * 1.9 * 4 * 2^-57 max|u|
-// beta plus a few roundings.  Fields whose exponent lies outside
-// [kVkEmaxLo, kVkEmaxHi] (all-zero or tiny fields, values near overflow, NaN,
-// Inf) take the FP64 form of vk_point_faces.
-constexpr int kVkEmaxLo = 120, kVkEmaxHi = 2030;
-
-__device__ __forceinline__ unsigned long long vk_face_sig(double c)
-{
-    // significand of c in [1, 2), its implicit bit included
-    return ((unsigned long long)__double_as_longlong(c) & 0x000fffffffffffffull) | 0x0010000000000000ull;
-}
-
-__device__ __forceinline__ bool vk_exact_ok(int emax) { return emax >= kVkEmaxLo && emax <= kVkEmaxHi; }
-
-// u' from the exact operator sums: one sum (all axes) rounded once on a cubic
-// grid, u' = fma(beta, D, u + dt f); else the three axis sums, each rounded
-// once, combined as the FP64 form combines them: (u + dt f) + ((bx Dx + by Dy)
-// + bz Dz).  C dU carries the scale 2^52 2^(1080 - e).
-template <bool CUBIC>
-__device__ __forceinline__ double vk_combine(double uc, double f, I128 dx, I128 dy, I128 dz, double bx, double by,
-                                             double bz, int emax)
-{
-    if constexpr (CUBIC) {
-        const double D = i128_to_double(i128_add(i128_add(dx, dy), dz), emax - 1132);
-        return __fma_rn(bx, D, __dadd_rn(uc, f));
-    } else {
-        const double Dx = i128_to_double(dx, emax - 1132), Dy = i128_to_double(dy, emax - 1132),
-                     Dz = i128_to_double(dz, emax - 1132);
-        return __dadd_rn(__dadd_rn(uc, f), __fma_rn(bz, Dz, __fma_rn(by, Dy, __dmul_rn(bx, Dx))));
-    }
-}
-
-// One update on the exact path from the seven u values (as doubles, the centre
-// also as its integer), the six face sums and dt f.
-template <bool CUBIC>
-__device__ __forceinline__ double vk_point_exact(double uc, long long Uc, long long Uxm, long long Uxp,
-                                                 long long Uym, long long Uyp, long long dzp, long long dzm,
-                                                 double cxm, double cxp, double cym, double cyp, double czm,
-                                                 double czp, double f, double bx, double by, double bz, int emax)
-{
-    const I128 dx = i128_sub(i128_mul(vk_face_sig(cxp), Uxp - Uc), i128_mul(vk_face_sig(cxm), Uc - Uxm));
-    const I128 dy = i128_sub(i128_mul(vk_face_sig(cyp), Uyp - Uc), i128_mul(vk_face_sig(cym), Uc - Uym));
-    const I128 dz = i128_sub(i128_mul(vk_face_sig(czp), dzp), i128_mul(vk_face_sig(czm), dzm));
-    return vk_combine<CUBIC>(uc, f, dx, dy, dz, bx, by, bz, emax);
-}
-
-// Interior (planes kbeg..kend-1) of an FP64 grid: the exact sums while the
-// field's exponent allows it, the FP64 form otherwise; every output joins the
-// step's maximum (slot (m3 + 1) % 3).  Every thread takes two consecutive x
-// points (16-byte loads of u, the face sums and dt f): four conversions per
-// point and half the load instructions of one point per thread, whose loads
-// left the kernel waiting on memory; three blocks per SM at 80 registers.
-// The products through the face between a thread's two points and through the
-// face below a plane (the face above it one plane earlier) are formed once: 9
-// products for two points instead of 12, and the sums stay exact, so the
-// result is the same.  Measured at 510^3: one point per thread 57 GLUP/s, two
-// points 77, shared fluxes 85; staging each plane through shared memory so
-// that every value is converted once (one block barrier per plane) 55, 71 with
-// the staging loads issued one plane ahead.  A thread whose second point is
-// the boundary node nx computes only the first.
-template <bool CUBIC>
-__global__ void __launch_bounds__(kVkBX* kVkBY, 3)
-    k_vk_interior_xs(const double* __restrict__ src, double* __restrict__ dst, const double* __restrict__ fc,
-                      const double* __restrict__ fdt, HeatGeom g, double bx, double by, double bz, int kbeg,
-                      int kend, int kchunk, FxState* fx, int m3)
-{
-    const int i0 = (blockIdx.x * kVkBX + threadIdx.x) * 2;
-    const int j = blockIdx.y * kVkBY + threadIdx.y;
-    const int k0 = kbeg + (int)blockIdx.z * kchunk;
-    const int k1 = min(k0 + kchunk, kend);
-    const int emax = xs_emax(fx, m3);
-    unsigned mx = 0;
-    if (i0 < g.nx && j < g.ny && k0 < k1) {
-        const bool two = i0 + 1 < g.nx;
-        const int64_t P = g.plane, Y = g.pitch;
-        const double* fxs = fc;
-        const double* fys = fc + g.total;
-        const double* fzs = fc + 2 * g.total;
-        auto ld2 = [](const double* p, double (&o)[2]) {
-            const double2 v = __ldg(reinterpret_cast<const double2*>(p));
-            o[0] = v.x;
-            o[1] = v.y;
-        };
-        int64_t c = g.at(i0, j, k0);
-        if (vk_exact_ok(emax)) {
-            // D = sum over faces of +- F, F = C (U beyond the face - U before it):
-            // the face between the thread's two points and the face below the
-            // plane (the face above the plane before) are each formed once
-            auto fix = [emax](double v) { return xs_fix(__double_as_longlong(v), emax); };
-            double uc[2], t[2], czm[2];
-            long long Uc[2];
-            I128 fzm[2];   // the flux through the face below plane k
-            ld2(src + c, uc);
-            ld2(src + c - P, t);
-            ld2(fzs + c - P, czm);
-#pragma unroll
-            for (int q = 0; q < 2; ++q) {
-                Uc[q] = fix(uc[q]);
-                fzm[q] = i128_mul(vk_face_sig(czm[q]), Uc[q] - fix(t[q]));
-            }
-            for (int k = k0; k < k1; ++k) {
-                double ua[2], ym[2], yp[2], cx[2], cym[2], cyp[2], cza[2], f[2];
-                ld2(src + c + P, ua);
-                ld2(src + c - Y, ym);
-                ld2(src + c + Y, yp);
-                ld2(fxs + c, cx);
-                ld2(fys + c - Y, cym);
-                ld2(fys + c, cyp);
-                ld2(fzs + c, cza);
-                ld2(fdt + c, f);
-                const long long Uxm = fix(__ldg(src + c - 1)), Uxp = fix(__ldg(src + c + 2));
-                const double cxm0 = __ldg(fxs + c - 1);
-                const I128 fa = i128_mul(vk_face_sig(cxm0), Uc[0] - Uxm);   // face i0 - 1/2
-                const I128 fb = i128_mul(vk_face_sig(cx[0]), Uc[1] - Uc[0]);  // face i0 + 1/2
-                const I128 fcx = i128_mul(vk_face_sig(cx[1]), Uxp - Uc[1]);  // face i0 + 3/2
-                long long Ua[2];
-                double v[2];
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    Ua[q] = fix(ua[q]);
-                    const I128 fzp = i128_mul(vk_face_sig(cza[q]), Ua[q] - Uc[q]);
-                    const I128 dx = q == 0 ? i128_sub(fb, fa) : i128_sub(fcx, fb);
-                    const I128 dy = i128_sub(i128_mul(vk_face_sig(cyp[q]), fix(yp[q]) - Uc[q]),
-                                             i128_mul(vk_face_sig(cym[q]), Uc[q] - fix(ym[q])));
-                    const I128 dz = i128_sub(fzp, fzm[q]);
-                    fzm[q] = fzp;
-                    v[q] = vk_combine<CUBIC>(uc[q], f[q], dx, dy, dz, bx, by, bz, emax);
-                }
-                if (two) {
-                    *reinterpret_cast<double2*>(dst + c) = make_double2(v[0], v[1]);
-                } else {
-                    dst[c] = v[0];
-                    v[1] = 0.0;
-                }
-#pragma unroll
-                for (int q = 0; q < 2; ++q) {
-                    const unsigned a = xs_abs_hi(v[q]);
-                    mx = a > mx ? a : mx;
-                    uc[q] = ua[q];
-                    Uc[q] = Ua[q];
-                }
-                c += P;
-            }
-        } else {
-            // outside the exact form's range: the FP64 form, point by point
-            for (int q = 0; q < (two ? 2 : 1); ++q) {
-                int64_t cq = c + q;
-                double u = __ldg(src + cq);
-                double dzmq = __dsub_rn(u, __ldg(src + cq - P));
-                double czmq = __ldg(fzs + cq - P);
-                for (int k = k0; k < k1; ++k) {
-                    const double ua = __ldg(src + cq + P), cza = __ldg(fzs + cq);
-                    const double dzp = __dsub_rn(ua, u);
-                    const double w = vk_point_faces(u, __ldg(src + cq - 1), __ldg(src + cq + 1), __ldg(src + cq - Y),
-                                                    __ldg(src + cq + Y), dzp, dzmq, __ldg(fxs + cq - 1), __ldg(fxs + cq),
-                                                    __ldg(fys + cq - Y), __ldg(fys + cq), czmq, cza, __ldg(fdt + cq),
-                                                    bx, by, bz);
-                    dst[cq] = w;
-                    const unsigned a = xs_abs_hi(w);
-                    mx = a > mx ? a : mx;
-                    u = ua;
-                    dzmq = dzp;
-                    czmq = cza;
-                    cq += P;
-                }
-            }
-        }
-    }
-    fx_finish<kVkBX * kVkBY>((unsigned long long)mx << 32, fx, m3, 0,
-                             blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0);
-}
-
-// Boundary planes 0 and nz-1 of an FP64 grid, as k_vk_interior_xs (one
-// point per thread).
-template <bool CUBIC>
-__global__ void __launch_bounds__(kVkBX* kVkBY)
-    k_vk_boundary_xs(const double* __restrict__ src, double* __restrict__ dst, const double* __restrict__ fc,
-                     const double* __restrict__ fdt, HeatGeom g, double bx, double by, double bz, FxState* fx,
-                     int m3)
-{
-    const int i = blockIdx.x * kVkBX + threadIdx.x;
-    const int j = blockIdx.y * kVkBY + threadIdx.y;
-    const int emax = xs_emax(fx, m3);
-    unsigned mx = 0;
-    if (i < g.nx && j < g.ny) {
-        const int k = (blockIdx.z == 0) ? 0 : g.nz - 1;
-        const int64_t P = g.plane, Y = g.pitch;
-        const int64_t c = g.at(i, j, k);
-        const double* fxs = fc;
-        const double* fys = fc + g.total;
-        const double* fzs = fc + 2 * g.total;
-        const double uc = __ldg(src + c);
-        double v;
-        if (vk_exact_ok(emax)) {
-            auto fix = [emax](double w) { return xs_fix(__double_as_longlong(w), emax); };
-            const long long Uc = fix(uc);
-            v = vk_point_exact<CUBIC>(uc, Uc, fix(__ldg(src + c - 1)), fix(__ldg(src + c + 1)),
-                                      fix(__ldg(src + c - Y)), fix(__ldg(src + c + Y)),
-                                      fix(__ldg(src + c + P)) - Uc, Uc - fix(__ldg(src + c - P)),
-                                      __ldg(fxs + c - 1), __ldg(fxs + c), __ldg(fys + c - Y), __ldg(fys + c),
-                                      __ldg(fzs + c - P), __ldg(fzs + c), __ldg(fdt + c), bx, by, bz, emax);
-        } else {
-            v = vk_point_faces(uc, __ldg(src + c - 1), __ldg(src + c + 1), __ldg(src + c - Y), __ldg(src + c + Y),
-                               __dsub_rn(__ldg(src + c + P), uc), __dsub_rn(uc, __ldg(src + c - P)),
-                               __ldg(fxs + c - 1), __ldg(fxs + c), __ldg(fys + c - Y), __ldg(fys + c),
-                               __ldg(fzs + c - P), __ldg(fzs + c), __ldg(fdt + c), bx, by, bz);
-        }
-        dst[c] = v;
-        mx = xs_abs_hi(v);
-    }
-    fx_finish<kVkBX * kVkBY>((unsigned long long)mx << 32, fx, m3, 0,
-                             blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0);
 }
 
 template <typename T>
@@ -384,7 +59,272 @@ __device__ __forceinline__ T vk_point(T uc, T uxm, T uxp, T uym, T uyp, T uzm, T
     return (uc + f) + ((bx * dx + by * dy) + bz * dz);
 }
 
-// FP32 Interior: every thread four consecutive x points (one 16-byte vector
+// ---- FP64, exact-sum form --------------------------------------------------
+// u' = (u + dt f) + beta D with D = sum over the faces of (kappa + kappa_nb)
+// (u_nb - u): the differences of the field's fixed-point integers (SH = 7: units
+// of 2^-60 of the field's largest binade) times the face sums in xs_flux, summed
+// in 64 bits, L = D 2^(1080 - e) to within 15 units of 4 2^-60 each rounded to a
+// double once.  One beta for every axis (a cubic grid) needs nothing more;
+// otherwise the axis sums are first scaled by beta_d / beta_max in 62-bit fixed
+// point.  The error against the formula in exact arithmetic is below 30 2^-57
+// max|u| beta plus a few roundings.  e is tracked per step in the handle's
+// FxState like the default FP64 arithmetic's.  Fields whose exponent lies outside
+// [kVkEmaxLo, kVkEmaxHi] (all-zero or tiny fields, values near overflow, NaN,
+// Inf) take vk_point.
+constexpr int kVkEmaxLo = 120, kVkEmaxHi = 2030;
+
+struct VkBeta {
+    double bx, by, bz;        // dt / (2 h_d^2)
+    double b;                 // the largest
+    int wh[3], wl[3];         // beta_d / b times 2^62, as xs_mulhi3 takes it
+    int exact;                // every kappa is in [0.5, 1)
+};
+
+__device__ __forceinline__ bool vk_exact_ok(int emax, double b)
+{
+    return emax >= max(kVkEmaxLo, xs_emax_lo(b)) && emax <= kVkEmaxHi;
+}
+
+// A block of 32 x 8 threads owns 64 x 8 columns and marches up its planes, every
+// thread two consecutive x points.  Each plane of the tile -- u and kappa with a
+// one-point halo, dt f without -- arrives by TMA into a ring of kVkNst stages, up
+// to kVkNst - 2 planes ahead of use; once plane k+1 lands, the block converts its
+// u in place (every thread its own two values, warps 0 and 1 the halo rows, warp
+// 2 the halo columns), so each value is converted once and no load waits on
+// memory inside the march.  The flux through the face between a thread's two
+// points and through the face below a plane are formed once.  One of a thread's
+// two points converts its sum on the FP64 pipe.  Every mbarrier wait is bounded,
+// as in heat_stream.cu.
+//
+// Instruction issue (62%), the FP64 pipe (57%) and DRAM (58%) share the time, 174
+// instructions per point.  510^3: 890 us per step, 149 GLUP/s = 4.77 TB/s of the
+// 32 bytes per update; 520 x 510 x 500 1176 us.  Before: face sums in three arrays
+// (48 bytes), their products summed in 128 bits, every neighbour converted where
+// it was used, 265 instructions: 1541 us and 2400 us.  Loads through L1 instead
+// of TMA: 1178 us.  Three resident blocks either way, but held to 80 registers
+// by the launch bound the compiler's schedule took 946 us; a 3-stage ring 1250,
+// 6 stages (two blocks) 1030; both points on the FP64 pipe 906, none 890.
+constexpr int kVkTW = 64, kVkBW = 68, kVkD = 2, kVkNst = 4;
+constexpr uint32_t kVkBoxBytes = (kVkBY + 2) * kVkBW * 8, kVkSrcBytes = kVkBY * kVkTW * 8;
+constexpr int kVkPlane = (int)((kVkBoxBytes + 127) / 128 * 128 / 8);   // words of a staged plane of u or kappa
+constexpr int kVkStage = 2 * kVkPlane + (int)(kVkSrcBytes / 8);        // u, kappa, dt f
+constexpr size_t kVkSmem = (size_t)kVkNst * (kVkStage * 8 + sizeof(uint64_t));
+
+template <bool CUBIC, bool EXACT>
+__device__ __forceinline__ unsigned vk_march(const CUtensorMap* umap, const CUtensorMap* kmap, const CUtensorMap* fmap,
+                                             double* __restrict__ dst, const HeatGeom& g, const VkBeta& B, int kb,
+                                             int ke, int emax, long long* stage, uint64_t* bars, int& s_abort, int* err)
+{
+    const int tx = threadIdx.x, ty = threadIdx.y, tid = ty * kVkBX + tx;
+    const int x0 = blockIdx.x * kVkTW, y0 = blockIdx.y * kVkBY;
+    const int X = x0 + 2 * tx, Y = y0 + ty;
+    const bool in = X < g.nx && Y < g.ny, two = X + 1 < g.nx;
+    const int own = (ty + 1) * kVkBW + kVkD + 2 * tx;
+    const int p_first = kb - 1, p_last = ke;
+    // converted besides the thread's own values: a pair of halo row 0 (warp 0) or
+    // 9 (warp 1), or one halo-column value (warp 2)
+    int extra = -1;
+    if (ty == 0) extra = kVkD + 2 * tx;
+    else if (ty == 1) extra = (kVkBY + 1) * kVkBW + kVkD + 2 * tx;
+    else if (ty == 2 && tx < 2 * kVkBY)
+        extra = tx < kVkBY ? (tx + 1) * kVkBW + kVkD - 1 : (tx - kVkBY + 1) * kVkBW + kVkD + kVkTW;
+    auto fix = [emax](long long b) -> long long { return EXACT ? xs_fix<7>(b, emax) : b; };
+    auto dbl = [](long long v) { return __longlong_as_double(v); };
+    const double r2 = EXACT ? xs_r2(B.b, emax) : 0.0;
+    auto issue = [&](int p, int slot) {   // plane p into its slot (thread 0)
+        long long* st = stage + slot * kVkStage;
+        mbar_arrive_expect_tx(&bars[slot], 2 * kVkBoxBytes + kVkSrcBytes);
+        tma_load_3d(st, umap, g.lead + x0 - kVkD, y0, p + 1, &bars[slot]);
+        tma_load_3d(st + kVkPlane, kmap, g.lead + x0 - kVkD, y0, p + 1, &bars[slot]);
+        tma_load_3d(st + 2 * kVkPlane, fmap, g.lead + x0, y0 + 1, p + 1, &bars[slot]);
+    };
+    // converts this thread's part of a staged plane; its own values before and after
+    auto convert = [&](long long* pl, double (&raw)[2], long long (&U)[2]) {
+        const longlong2 v = *reinterpret_cast<const longlong2*>(pl + own);
+        raw[0] = dbl(v.x);
+        raw[1] = dbl(v.y);
+        U[0] = fix(v.x);
+        U[1] = fix(v.y);
+        if constexpr (EXACT) {
+            *reinterpret_cast<longlong2*>(pl + own) = make_longlong2(U[0], U[1]);
+            if (ty < 2) {
+                const longlong2 h = *reinterpret_cast<const longlong2*>(pl + extra);
+                *reinterpret_cast<longlong2*>(pl + extra) = make_longlong2(fix(h.x), fix(h.y));
+            } else if (extra >= 0) {
+                pl[extra] = fix(pl[extra]);
+            }
+        }
+    };
+
+    int issued = p_first - 1, drain_from = p_first;
+    if (tid == 0)
+        for (int s = 0; s < kVkNst && p_first + s <= p_last; ++s) {
+            issue(p_first + s, s);
+            issued = p_first + s;
+        }
+    unsigned mx = 0;
+    double uc[2], un[2];
+    long long Uc[2], Un[2], kc[2], fb[2] = {0, 0};
+    bool ok = mbar_wait_bounded(&bars[0], 0) && mbar_wait_bounded(&bars[1], 0);
+    {
+        const longlong2 ub = *reinterpret_cast<const longlong2*>(stage + own);
+        const longlong2 kl = *reinterpret_cast<const longlong2*>(stage + kVkPlane + own);
+        const longlong2 kv = *reinterpret_cast<const longlong2*>(stage + kVkStage + kVkPlane + own);
+        kc[0] = kv.x;
+        kc[1] = kv.y;
+        convert(stage + kVkStage, uc, Uc);
+        if constexpr (EXACT) {   // the flux through the face below the first plane
+            fb[0] = xs_flux(kl.x, kc[0], Uc[0] - fix(ub.x));
+            fb[1] = xs_flux(kl.y, kc[1], Uc[1] - fix(ub.y));
+            fence_proxy_async_smem();   // before the barrier after which TMA may refill the slot
+        }
+    }
+    if (!ok) {
+        atomicExch(err, 1);
+        s_abort = 1;
+    }
+    __syncthreads();
+    int s_cur = 1, n_cur = 0;
+    double* out = dst + g.at(in ? X : 0, in ? Y : 0, kb);
+    if (!s_abort) {
+        for (int k = kb; k < ke; ++k) {
+            const int s_nxt = s_cur + 1 == kVkNst ? 0 : s_cur + 1, s_prev = s_cur == 0 ? kVkNst - 1 : s_cur - 1;
+            const int n_nxt = s_nxt == 0 ? n_cur + 1 : n_cur;
+            if (!mbar_wait_bounded(&bars[s_nxt], (uint32_t)n_nxt & 1u)) {
+                atomicExch(err, 1);
+                s_abort = 1;
+            }
+            convert(stage + s_nxt * kVkStage, un, Un);
+            const long long* pu = stage + s_cur * kVkStage + own;
+            const long long* pk = pu + kVkPlane;
+            const longlong2 kav = *reinterpret_cast<const longlong2*>(stage + s_nxt * kVkStage + kVkPlane + own);
+            const longlong2 kym = *reinterpret_cast<const longlong2*>(pk - kVkBW);
+            const longlong2 kyp = *reinterpret_cast<const longlong2*>(pk + kVkBW);
+            const longlong2 uym = *reinterpret_cast<const longlong2*>(pu - kVkBW);
+            const longlong2 uyp = *reinterpret_cast<const longlong2*>(pu + kVkBW);
+            const double2 f = *reinterpret_cast<const double2*>(stage + s_cur * kVkStage + 2 * kVkPlane + ty * kVkTW +
+                                                                2 * tx);
+            const long long Ul = pu[-1], Ur = pu[2], kl = pk[-1], kr = pk[2];
+            double w[2];
+            if constexpr (EXACT) {
+                const long long fl = xs_flux(kl, kc[0], Uc[0] - Ul);
+                const long long fm = xs_flux(kc[0], kc[1], Uc[1] - Uc[0]);
+                const long long fr = xs_flux(kc[1], kr, Ur - Uc[1]);
+#pragma unroll
+                for (int q = 0; q < 2; ++q) {
+                    const long long fa = xs_flux(kc[q], q ? kav.y : kav.x, Un[q] - Uc[q]);
+                    const long long dx = q == 0 ? fm - fl : fr - fm;
+                    const long long dy = xs_flux(kc[q], q ? kyp.y : kyp.x, (q ? uyp.y : uyp.x) - Uc[q]) -
+                                         xs_flux(kc[q], q ? kym.y : kym.x, Uc[q] - (q ? uym.y : uym.x));
+                    const long long dz = fa - fb[q];
+                    fb[q] = fa;
+                    const long long L = CUBIC ? dx + dy + dz
+                                              : xs_mulhi3(dx << 2, B.wh[0], B.wl[0]) + xs_mulhi3(dy << 2, B.wh[1], B.wl[1]) +
+                                                    xs_mulhi3(dz << 2, B.wh[2], B.wl[2]);
+                    const double uf = __dadd_rn(uc[q], q ? f.y : f.x);
+                    w[q] = q == 0 ? xs_apply<true>(uf, L, B.b, r2, emax) : xs_apply<false>(uf, L, B.b, r2, emax);
+                }
+            } else {
+                const long long* pb = stage + s_prev * kVkStage + own;
+                const longlong2 ub = *reinterpret_cast<const longlong2*>(pb);
+                const longlong2 kbv = *reinterpret_cast<const longlong2*>(pb + kVkPlane);
+#pragma unroll
+                for (int q = 0; q < 2; ++q)
+                    w[q] = vk_point<double>(uc[q], q ? uc[0] : dbl(Ul), q ? dbl(Ur) : uc[1], dbl(q ? uym.y : uym.x),
+                                            dbl(q ? uyp.y : uyp.x), dbl(q ? ub.y : ub.x), un[q], dbl(kc[q]),
+                                            dbl(q ? kc[0] : kl), dbl(q ? kr : kc[1]), dbl(q ? kym.y : kym.x),
+                                            dbl(q ? kyp.y : kyp.x), dbl(q ? kbv.y : kbv.x), dbl(q ? kav.y : kav.x),
+                                            q ? f.y : f.x, B.bx, B.by, B.bz);
+            }
+            if (in) {
+                if (two) {
+                    *reinterpret_cast<double2*>(out) = make_double2(w[0], w[1]);
+                } else {
+                    out[0] = w[0];
+                    w[1] = 0.0;
+                }
+                mx = max(mx, max(xs_abs_hi(w[0]), xs_abs_hi(w[1])));
+            }
+#pragma unroll
+            for (int q = 0; q < 2; ++q) {
+                uc[q] = un[q];
+                Uc[q] = Un[q];
+            }
+            kc[0] = kav.x;
+            kc[1] = kav.y;
+            out += g.plane;
+            if constexpr (EXACT) fence_proxy_async_smem();
+            __syncthreads();
+            if (s_abort) {
+                drain_from = k + 1;
+                break;
+            }
+            if (tid == 0 && issued < p_last) {   // plane k-1's slot is free
+                fence_proxy_async_smem();
+                issue(issued + 1, s_prev);
+                ++issued;
+            }
+            s_cur = s_nxt;
+            n_cur = n_nxt;
+        }
+    }
+    if (s_abort && tid == 0) {
+        const long long t0 = clock64();   // one time budget for the whole drain
+        for (int p = drain_from; p <= issued; ++p) {
+            const int i = p - p_first;
+            if (!mbar_wait_until(&bars[i % kVkNst], (uint32_t)(i / kVkNst) & 1u, t0, kWaitCycles)) {
+                atomicExch(err, 2);   // loads may still be landing: the context is suspect
+                break;
+            }
+        }
+    }
+    return mx;
+}
+
+template <bool CUBIC>
+__global__ void __launch_bounds__(kVkBX* kVkBY, 2)
+    k_vk_xs(const __grid_constant__ CUtensorMap umap, const __grid_constant__ CUtensorMap kmap,
+            const __grid_constant__ CUtensorMap fmap, double* __restrict__ dst, HeatGeom g, VkBeta B, int kbeg, int kend,
+            int kchunk, FxState* fx, int m3, int* err)
+{
+    extern __shared__ __align__(128) unsigned char smem_raw[];
+    long long* stage = reinterpret_cast<long long*>(smem_raw);
+    uint64_t* bars = reinterpret_cast<uint64_t*>(stage + kVkNst * kVkStage);
+    __shared__ int s_abort;
+    if (threadIdx.x == 0 && threadIdx.y == 0) {
+        // a block that starts after another one gave up does no work at all
+        s_abort = *(volatile int*)err;
+        for (int s = 0; s < kVkNst; ++s) mbar_init(&bars[s], 1);
+        fence_mbar_init();
+    }
+    __syncthreads();
+    if (s_abort) return;
+    const int kb = kbeg + (int)blockIdx.z * kchunk;
+    const int ke = min(kb + kchunk, kend);
+    const int emax = xs_emax(fx, m3);
+    const unsigned mx =
+        B.exact && vk_exact_ok(emax, B.b)
+            ? vk_march<CUBIC, true>(&umap, &kmap, &fmap, dst, g, B, kb, ke, emax, stage, bars, s_abort, err)
+            : vk_march<CUBIC, false>(&umap, &kmap, &fmap, dst, g, B, kb, ke, emax, stage, bars, s_abort, err);
+    if (s_abort) return;   // uniform: every thread passed the barrier that saw it
+    fx_finish<kVkBX * kVkBY>((unsigned long long)mx << 32, fx, m3, 0,
+                             blockIdx.x == 0 && blockIdx.y == 0 && blockIdx.z == 0);
+}
+
+// The tensor maps of an FP64 handle: its two buffers, kappa, dt f.
+int vk_maps(CUtensorMap (&maps)[4], void* const (&buf)[2], void* kap, void* fdt, const HeatGeom& g)
+{
+    void* const base[4] = {buf[0], buf[1], kap, fdt};
+    for (int i = 0; i < 4; ++i) {
+        const int e = encode_field_map(&maps[i], base[i], CU_TENSOR_MAP_DATA_TYPE_INT64, sizeof(double),
+                                       (uint64_t)g.pitch, (uint64_t)(g.ny + 2), (uint64_t)(g.nz + 2),
+                                       i < 3 ? kVkBW : kVkTW, i < 3 ? kVkBY + 2 : kVkBY);
+        if (e != 0) return e;
+    }
+    return 0;
+}
+
+// FP32: every thread four consecutive x points (one 16-byte vector
 // of u, kappa and dt f per row), so a point costs about 3.5 load instructions
 // instead of 11; the update of each point is vk_point's.  A thread whose four
 // points run past nx loads element by element up to the boundary node nx (u
@@ -393,7 +333,7 @@ __device__ __forceinline__ T vk_point(T uc, T uxm, T uxp, T uym, T uyp, T uzm, T
 // registers, with 8-plane chunks, ran 340 GLUP/s at 510^3 against 265 with
 // three blocks at 80 registers.
 __global__ void __launch_bounds__(kVkBX* kVkBY, 4)
-    k_vk_interior_f4(const float* __restrict__ src, float* __restrict__ dst, const float* __restrict__ kap,
+    k_vk_f4(const float* __restrict__ src, float* __restrict__ dst, const float* __restrict__ kap,
                      const float* __restrict__ fdt, HeatGeom g, float bx, float by, float bz, int kbeg, int kend,
                      int kchunk)
 {
@@ -461,91 +401,60 @@ __global__ void __launch_bounds__(kVkBX* kVkBY, 4)
     }
 }
 
-template <typename T>
-__global__ void __launch_bounds__(kVkBX* kVkBY)
-    k_vk_boundary(const T* __restrict__ src, T* __restrict__ dst, const T* __restrict__ kap,
-                  const T* __restrict__ fdt, HeatGeom g, T bx, T by, T bz)
-{
-    const int i = blockIdx.x * kVkBX + threadIdx.x;
-    const int j = blockIdx.y * kVkBY + threadIdx.y;
-    if (i >= g.nx || j >= g.ny) return;
-    const int k = (blockIdx.z == 0) ? 0 : g.nz - 1;
-    const int64_t P = g.plane, Y = g.pitch;
-    const int64_t c = g.at(i, j, k);
-    dst[c] = vk_point<T>(__ldg(src + c), __ldg(src + c - 1), __ldg(src + c + 1), __ldg(src + c - Y),
-                         __ldg(src + c + Y), __ldg(src + c - P), __ldg(src + c + P), __ldg(kap + c),
-                         __ldg(kap + c - 1), __ldg(kap + c + 1), __ldg(kap + c - Y), __ldg(kap + c + Y),
-                         __ldg(kap + c - P), __ldg(kap + c + P), __ldg(fdt + c), bx, by, bz);
-}
-
 int vk_init(const VkCall& c, double dt)
 {
     const int64_t n = (int64_t)(c.g->nx + 2) * (c.g->ny + 2) * (c.g->nz + 2);
     int64_t blocks = (n + 255) / 256;
     if (blocks > (int64_t)kNumSMs * 16) blocks = (int64_t)kNumSMs * 16;
     if (c.f64)
-        k_vk_init_faces<<<(unsigned)blocks, 256, 0, c.stream>>>((double*)c.kap, (double*)c.fdt, *c.g, dt,
-                                                                c.face_off);
+        k_vk_init<double><<<(unsigned)blocks, 256, 0, c.stream>>>((double*)c.kap, (double*)c.fdt, *c.g, dt, c.kappa_off);
     else
-        k_vk_init<float><<<(unsigned)blocks, 256, 0, c.stream>>>((float*)c.kap, (float*)c.fdt, *c.g, dt);
+        k_vk_init<float><<<(unsigned)blocks, 256, 0, c.stream>>>((float*)c.kap, (float*)c.fdt, *c.g, dt, nullptr);
     HS_CHECK_LAUNCH("heat: kappa/source init kernel");
     return HS_OK;
 }
 
-template <typename T>
-int vk_launch_t(const VkCall& c)
+int vk_launch(const VkCall& c)
 {
     const HeatGeom& g = *c.g;
-    dim3 block(kVkBX, kVkBY, 1);
-    const T bx = (T)c.bx, by = (T)c.by, bz = (T)c.bz;
-    constexpr bool kFaces = std::is_same<T, double>::value;
-    if (c.part == 0) {
-        if (g.nz < 3) return HS_OK;
-        const int kbeg = 1, kend = g.nz - 1;
-        const int nchunks = (kend - kbeg + c.kchunk - 1) / c.kchunk;
-        dim3 grid((g.nx + kVkBX - 1) / kVkBX, (g.ny + kVkBY - 1) / kVkBY, nchunks);
-        if constexpr (kFaces) {
-            if (c.fx) {
-                dim3 grid2((g.nx + 2 * kVkBX - 1) / (2 * kVkBX), grid.y, grid.z);
-                auto kern = (bx == by && by == bz) ? k_vk_interior_xs<true> : k_vk_interior_xs<false>;
-                kern<<<grid2, block, 0, c.stream>>>((const double*)c.src, (double*)c.dst, (const double*)c.kap,
-                                                    (const double*)c.fdt, g, bx, by, bz, kbeg, kend, c.kchunk,
-                                                    c.fx, c.m3);
-            }
-            else
-                k_vk_interior_faces<<<grid, block, 0, c.stream>>>((const double*)c.src, (double*)c.dst,
-                                                                  (const double*)c.kap, (const double*)c.fdt, g,
-                                                                  bx, by, bz, kbeg, kend, c.kchunk);
+    if (c.kend <= c.kbeg) return HS_OK;
+    const int nchunks = (c.kend - c.kbeg + c.kchunk - 1) / c.kchunk;
+    const dim3 block(kVkBX, kVkBY, 1);
+    const unsigned by = (g.ny + kVkBY - 1) / kVkBY;
+    if (c.f64) {
+        VkBeta B;
+        B.bx = c.bx;
+        B.by = c.by;
+        B.bz = c.bz;
+        B.b = std::fmax(c.bx, std::fmax(c.by, c.bz));
+        const double axis[3] = {c.bx, c.by, c.bz};
+        for (int d = 0; d < 3; ++d) {
+            const long long w = B.b > 0.0 ? std::llrint(std::ldexp(axis[d] / B.b, 62)) : 0ll;
+            B.wl[d] = (int)(unsigned)w;
+            B.wh[d] = (int)((w - B.wl[d]) >> 32);
         }
-        else {
-            dim3 grid4((g.nx + 4 * kVkBX - 1) / (4 * kVkBX), grid.y, grid.z);
-            k_vk_interior_f4<<<grid4, block, 0, c.stream>>>((const float*)c.src, (float*)c.dst,
-                                                            (const float*)c.kap, (const float*)c.fdt, g,
-                                                            (float)bx, (float)by, (float)bz, kbeg, kend,
-                                                            c.kchunk);
-        }
-        HS_CHECK_LAUNCH("heat variable-kappa interior kernel");
+        B.exact = c.exact;
+        const bool cubic = c.bx == c.by && c.by == c.bz;
+        auto kern = cubic ? k_vk_xs<true> : k_vk_xs<false>;
+        // once per process, under the thread-safe initialisation of a local static
+        static const cudaError_t configured = [] {
+            const cudaError_t e = cudaFuncSetAttribute(k_vk_xs<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kVkSmem);
+            return e != cudaSuccess ? e
+                                    : cudaFuncSetAttribute(k_vk_xs<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                                           (int)kVkSmem);
+        }();
+        HS_TRY_CUDA(configured, "heat: variable-kappa kernel smem attribute");
+        const dim3 grid((g.nx + kVkTW - 1) / kVkTW, by, nchunks);
+        kern<<<grid, block, kVkSmem, c.stream>>>(*c.umap, *c.kmap, *c.fmap, (double*)c.dst, g, B, c.kbeg, c.kend, c.kchunk,
+                                                 c.fx, c.m3, c.err);
     } else {
-        dim3 grid((g.nx + kVkBX - 1) / kVkBX, (g.ny + kVkBY - 1) / kVkBY, g.nz >= 2 ? 2 : 1);
-        if constexpr (kFaces) {
-            if (c.fx) {
-                auto kern = (bx == by && by == bz) ? k_vk_boundary_xs<true> : k_vk_boundary_xs<false>;
-                kern<<<grid, block, 0, c.stream>>>((const double*)c.src, (double*)c.dst, (const double*)c.kap,
-                                                   (const double*)c.fdt, g, bx, by, bz, c.fx, c.m3);
-            }
-            else
-                k_vk_boundary_faces<<<grid, block, 0, c.stream>>>((const double*)c.src, (double*)c.dst,
-                                                                  (const double*)c.kap, (const double*)c.fdt, g,
-                                                                  bx, by, bz);
-        }
-        else
-            k_vk_boundary<T><<<grid, block, 0, c.stream>>>((const T*)c.src, (T*)c.dst, (const T*)c.kap,
-                                                           (const T*)c.fdt, g, bx, by, bz);
-        HS_CHECK_LAUNCH("heat variable-kappa boundary kernel");
+        const dim3 grid((g.nx + 4 * kVkBX - 1) / (4 * kVkBX), by, nchunks);
+        k_vk_f4<<<grid, block, 0, c.stream>>>((const float*)c.src, (float*)c.dst, (const float*)c.kap,
+                                                       (const float*)c.fdt, g, (float)c.bx, (float)c.by, (float)c.bz,
+                                                       c.kbeg, c.kend, c.kchunk);
     }
+    HS_CHECK_LAUNCH("heat variable-kappa kernel");
     return HS_OK;
 }
-
-int vk_launch(const VkCall& c) { return c.f64 ? vk_launch_t<double>(c) : vk_launch_t<float>(c); }
 
 }  // namespace hcg

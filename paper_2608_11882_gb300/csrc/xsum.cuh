@@ -45,18 +45,21 @@ __device__ __forceinline__ double xs_r2(double r, int emax)
 }
 
 // The fixed-point integer of the double with bit pattern `bits` (its exponent
-// field must not exceed emax): the mantissa with its implicit bit, times 2^5,
+// field must not exceed emax): the mantissa with its implicit bit, times 2^SH,
 // in ones' complement for negative values, shifted right arithmetically by
-// emax - e (at most 63) -- floor((u 2^(1080 - emax)) - [u < 0] 2^-t), within two
-// units of u 2^(1080 - emax).  Zeros and subnormals give 0 or -1 for emax >= 64.
+// emax - e (at most 63) -- floor((u 2^(1075 + SH - emax)) - [u < 0] 2^-t), within
+// two units of u 2^(1075 + SH - emax).  Zeros and subnormals give 0 or -1 for
+// emax >= 64.
+template <int SH = 5>
 __device__ __forceinline__ long long xs_fix(long long bits, int emax)
 {
     const unsigned hi = (unsigned)((unsigned long long)bits >> 32), lo = (unsigned)bits;
     const unsigned s = (unsigned)((int)hi >> 31);   // 0 or all ones
     const unsigned e = (hi >> 20) & 0x7ffu;
     const unsigned t = min((unsigned)(emax - (int)e), 63u);
-    const unsigned mh = ((__funnelshift_l(lo, hi, 5) & 0x01ffffffu) | 0x02000000u) ^ s;
-    const unsigned ml = (lo << 5) ^ s;
+    constexpr unsigned one = 1u << (20 + SH);   // the implicit bit
+    const unsigned mh = ((__funnelshift_l(lo, hi, SH) & (one - 1u)) | one) ^ s;
+    const unsigned ml = (lo << SH) ^ s;
     return (long long)(((unsigned long long)mh << 32) | ml) >> t;
 }
 
@@ -100,66 +103,27 @@ __device__ __forceinline__ double xs_apply(double uc, long long L, double r, dou
     return __fma_rn(r, xs_unfix(L, emax), uc);
 }
 
-// ---- exact weighted sums: 128-bit arithmetic -----------------------------
-// A sum of products C d, C < 2^53 an integer weight and d a difference of two
-// fixed-point values (|d| < 2^60), is exact in 128-bit two's complement
-// (hi:lo) for up to 2^14 terms; it is rounded once to FP64 by i128_to_double.
-struct I128 {
-    unsigned long long lo;
-    long long hi;
-};
-
-// C d as a 128-bit value, exactly.
-__device__ __forceinline__ I128 i128_mul(unsigned long long C, long long d)
+// ---- weighted differences -------------------------------------------------
+// d w / 2^64 to within 2.5 units, w = hi 2^32 + lo with a signed low part and
+// 0 <= hi < 2^31: the three 32-bit products that reach the high word.
+__device__ __forceinline__ long long xs_mulhi3(long long d, int hi, int lo)
 {
-    return I128{(unsigned long long)d * C, __mul64hi(d, (long long)C)};
+    const int dh = (int)(d >> 32);
+    return (long long)dh * hi + __mulhi(dh, lo) + (long long)__umulhi((unsigned)d, (unsigned)hi);
 }
 
-// a + b and a - b, exactly (two's complement, no overflow within the callers' ranges).
-__device__ __forceinline__ I128 i128_add(I128 a, I128 b)
+// The flux c d through a face: d the difference of two values' integers with
+// SH = 7 (|d| < 2^61, so units of u 2^(1082 - emax)), c in [1, 2) the sum of two
+// coefficients in [0.5, 1), given as their bit patterns.  Returns c d / 4 to
+// within 2.5 units, c as the 63-bit integer c 2^62 (exact: the sum of the two
+// 53-bit significands, shifted).  Six of them sum without overflow (below
+// 6 1.9/4 2^61), in units of u 2^(1080 - emax).
+__device__ __forceinline__ long long xs_flux(long long ca, long long cb, long long d)
 {
-    asm("add.cc.u64 %0, %0, %2;\n\taddc.u64 %1, %1, %3;" : "+l"(a.lo), "+l"(a.hi) : "l"(b.lo), "l"(b.hi));
-    return a;
-}
-__device__ __forceinline__ I128 i128_sub(I128 a, I128 b)
-{
-    asm("sub.cc.u64 %0, %0, %2;\n\tsubc.u64 %1, %1, %3;" : "+l"(a.lo), "+l"(a.hi) : "l"(b.lo), "l"(b.hi));
-    return a;
-}
-
-// (hi:lo) 2^s rounded to the nearest double, ties to even.  The caller keeps
-// |hi:lo| < 2^120 and s such that every nonzero result is a normal number.
-__device__ __forceinline__ double i128_to_double(I128 a, int s)
-{
-    const unsigned long long sign = (unsigned long long)(a.hi >> 63);
-    unsigned long long mlo, mhi;   // |hi:lo|
-    if (sign) {
-        mlo = 0ull - a.lo;
-        mhi = ~(unsigned long long)a.hi + (a.lo == 0ull ? 1ull : 0ull);
-    } else {
-        mlo = a.lo;
-        mhi = (unsigned long long)a.hi;
-    }
-    if ((mhi | mlo) == 0ull) return 0.0;
-    const int lz = mhi ? __clzll((long long)mhi) : 64 + __clzll((long long)mlo);   // >= 8
-    // the magnitude shifted left by lz - 1: its leading one at bit 126, so the
-    // top 64 bits n hold it at bit 62; the bits below join n's bit 0 (sticky)
-    const int t = lz - 1;
-    unsigned long long n, rest;
-    if (t >= 64) {
-        n = mlo << (t - 64);
-        rest = 0ull;
-    } else {
-        n = (mhi << t) | (mlo >> (64 - t));   // t >= 7, so 64 - t < 64
-        rest = mlo << t;
-    }
-    n |= rest != 0ull ? 1ull : 0ull;
-    const unsigned long long q = (n + 0x1ffull + ((n >> 10) & 1ull)) >> 10;   // 2^52 <= q <= 2^53
-    // the leading one is bit p = 127 - lz of the magnitude: biased exponent
-    // p + s + 1023; q's bit 52 (or a carry to 53) adds into the exponent field
-    const long long e1 = (long long)(127 - lz + s + 1022);
-    const unsigned long long bits = ((unsigned long long)e1 << 52) + q + (sign << 63);
-    return __longlong_as_double((long long)bits);
+    const unsigned long long s = (unsigned long long)(ca + cb) << 9;   // bits 0..52 of the sum, the exponents above
+    const int lo = (int)(unsigned)s;
+    const int hi = (int)(((unsigned)(s >> 32) & 0x3fffffffu) | 0x40000000u) + (int)((unsigned)lo >> 31);
+    return xs_mulhi3(d, hi, lo);
 }
 
 // |u| of a result as the high word of its bit pattern (the exponent field and
