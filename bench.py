@@ -72,7 +72,9 @@ HEAT_MODES = {
 #    32 B (FP64) / 16 B (FP32) per update;
 #  * CG per unknown and iteration: SpMV 16 B (read p, write q), x/r update 48 B
 #    (read x, p, r, q; write x, r), p update 24 B (read r, p; write p) = 88 B
-#    matrix-free; CSR adds 12 B per stored entry and 4 B of row pointer per row;
+#    matrix-free; CSR adds 12 B per stored entry and 4 B of row pointer per row
+#    (the textbook passes: the solver itself moves 76 to 80 B, x added where its
+#    direction is read anyway);
 #  * mixed-precision CG per inner iteration and unknown: matrix-free (nx a multiple
 #    of 4), the p update folded into the SpMV 16 B (read r, p; write p', q) and the
 #    update 24 B = 40 B; CSR: SpMV 8 B + 8 B per entry and 4 B per row, update 24 B,

@@ -109,6 +109,7 @@ __global__ void __launch_bounds__(kCgBlock)
             S->done = 2;   // breakdown: A is not positive definite on p
         } else {
             S->alpha = S->rho / tot;
+            S->alpha2[S->iters & 1] = S->alpha;
         }
     }
 }
@@ -134,22 +135,21 @@ __global__ void __launch_bounds__(kSpBlock, kSpMinBlocks)
             S->done = 2;   // breakdown: A is not positive definite on p
         } else {
             S->alpha = S->rho / tot;
+            S->alpha2[S->iters & 1] = S->alpha;
         }
     }
 }
 
-// x += alpha p, r -= alpha q fused with r.r; the last block tests convergence
+// r -= alpha q fused with r.r; the last block tests convergence
 // and forms beta.
 __global__ void __launch_bounds__(kCgBlock)
-    k_cg_update(int64_t n, double* __restrict__ x, double* __restrict__ r,
-                const double* __restrict__ p, const double* __restrict__ q, double* partials,
-                CgScalars* S)
+    k_cg_update(int64_t n, double* __restrict__ r, const double* __restrict__ q, double* partials, CgScalars* S)
 {
     grid_dependency_wait();
     if (*(volatile int32_t*)&S->done) return;
     __shared__ double sh[kCgBlock / 32];
     const double alpha = S->alpha;
-    const double rr = cg_update_rows(n, x, r, p, q, alpha, (int64_t)blockIdx.x * kCgBlock + threadIdx.x,
+    const double rr = cg_update_rows(n, r, q, alpha, (int64_t)blockIdx.x * kCgBlock + threadIdx.x,
                                      (int64_t)gridDim.x * kCgBlock);
     allow_dependents();
     const double blk = block_sum<kCgBlock>(rr, sh);
@@ -168,19 +168,35 @@ __global__ void __launch_bounds__(kCgBlock)
     }
 }
 
-// p = r + beta p.
+// The direction pass of iteration `it`: p' = r + beta p unless the solve has
+// stopped, and x for the iterations not added to it yet -- with two direction
+// buffers (pn another buffer than p) every second iteration's, else this one's.
+// `last`: no iteration follows.  A pass enqueued past the stop does nothing.
 __global__ void __launch_bounds__(kCgBlock)
-    k_cg_pupdate(int64_t n, const double* __restrict__ r, double* __restrict__ p, CgScalars* S,
-                 int track_pmax)
+    k_cg_direction(int64_t n, const double* r, const double* p, double* pn, double* x, CgScalars* S, int track_pmax,
+                   int it, int last)
 {
     grid_dependency_wait();
-    if (*(volatile int32_t*)&S->done) return;
-    const double beta = S->beta;
-    const unsigned pm = cg_pupdate_rows(n, r, p, beta, (int64_t)blockIdx.x * kCgBlock + threadIdx.x,
-                                        (int64_t)gridDim.x * kCgBlock);
+    const int iters = *(volatile int32_t*)&S->iters, done = *(volatile int32_t*)&S->done;
+    const bool next = done == 0 && !last;
+    const double alpha = S->alpha2[it & 1], alpha0 = S->alpha2[(it + 1) & 1], beta = S->beta;
+    const int64_t t0 = (int64_t)blockIdx.x * kCgBlock + threadIdx.x, stride = (int64_t)gridDim.x * kCgBlock;
+    if (iters != it + 1) {
+        // a breakdown in this iteration's SpMV leaves the iteration before it to be added
+        if (done == 2 && iters == it && pn != p && (it & 1))
+            (void)cg_direction_rows<X_ONE>(n, r, pn, nullptr, pn, x, alpha0, 0.0, 0.0, false, t0, stride);
+        return;
+    }
+    unsigned pm;
+    if (pn != p && (it & 1))   // pn holds the direction before p
+        pm = cg_direction_rows<X_TWO>(n, r, p, pn, pn, x, alpha, alpha0, beta, next, t0, stride);
+    else if (pn == p || !next)
+        pm = cg_direction_rows<X_ONE>(n, r, p, nullptr, pn, x, alpha, 0.0, beta, next, t0, stride);
+    else
+        pm = cg_direction_rows<X_NONE>(n, r, p, nullptr, pn, x, alpha, 0.0, beta, next, t0, stride);
     allow_dependents();
-    // the update kernel has counted this iteration: p is the next one's direction
-    if (track_pmax) cg_fold_pmax(pm, S, S->iters % 3, blockIdx.x == 0);
+    // the update kernel has counted this iteration: pn is the next one's direction
+    if (track_pmax && next) cg_fold_pmax(pm, S, (it + 1) % 3, blockIdx.x == 0);
 }
 
 // Largest |p| high word into S->pmax[0] (the direction's scale the
@@ -426,13 +442,15 @@ int cg_create_vectors(hs_cg_t* out, const hs_op* A, void* stream, bool need_p)
     auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t s_ctl = align(sizeof(CgSmallCtl)), s_part = align(sizeof(double) * cg_partials(c->A, c->grid));
     const size_t s_vec = align(sizeof(double) * (size_t)cg_vector_len(c->A));
-    CG_ALLOC(c->arena, s_ctl + s_part + (need_p ? 3 : 2) * s_vec);
+    const bool two = need_p && cg_two_directions(c->A);
+    CG_ALLOC(c->arena, s_ctl + s_part + (two ? 4 : need_p ? 3 : 2) * s_vec);
     c->ctl = (char*)c->arena;
     c->S = &((CgSmallCtl*)c->ctl)->S;
     c->partials = (double*)(c->ctl + s_ctl);
     c->r = (double*)(c->ctl + s_ctl + s_part);
     c->q = (double*)(c->ctl + s_ctl + s_part + s_vec);
     c->p = need_p ? (double*)(c->ctl + s_ctl + s_part + 2 * s_vec) : nullptr;
+    c->p2 = two ? (double*)(c->ctl + s_ctl + s_part + 3 * s_vec) : nullptr;
     // the host mirror of the scalars: ordinary memory (pinned memory would
     // cost a device-wide synchronisation to allocate and to free)
     c->S_host = new (std::nothrow) CgScalars();
@@ -576,11 +594,18 @@ int cg_run(hs_cg_t c, const void* b_in, void* x_inout, int host_buffers, double 
     const int track = mode == SP_STAGED;   // the staged SpMV needs p's largest exponent
     const int shares = mode == SP_STAGED ? spmv_shares(c->grid) : c->grid;
     // the staged SpMV takes p through TMA when the grid and the vectors allow
-    CUtensorMap pmap;
+    double* const dir[2] = {c->p, c->p2 ? c->p2 : c->p};   // the direction of iteration i is in dir[i % 2]
+    CUtensorMap pmap[2];
     const bool tma = mode == SP_STAGED && spmv_tma_eligible(c->A, c->p, c->q, c->grid) &&
-                     spmv_tma_map(&pmap, c->A, c->p) == 0;
+                     spmv_tma_map(&pmap[0], c->A, dir[0]) == 0 && spmv_tma_map(&pmap[1], c->A, dir[1]) == 0;
     k_cg_start<<<c->grid, kCgBlock, 0, c->stream>>>(n, b, c->q, c->r, c->p, c->partials, c->S, track);
     HS_CHECK_LAUNCH("cg: start kernel");
+
+    // The direction pass takes four blocks per SM: 243 us per iteration at 256^3,
+    // against 268 with the other passes' eight, whose streams lie further apart in
+    // DRAM, and 257 with 64 short ones, whose reads of the scalars weigh more (the
+    // update pass, bound by its FP64 instructions, keeps eight: 250 with four).
+    const int dgrid = std::min(c->grid, kNumSMs * 4);
 
     // Iterate in chunks, reading the stop flag and count between chunks.
     int32_t enqueued = 0;
@@ -594,31 +619,34 @@ int cg_run(hs_cg_t c, const void* b_in, void* x_inout, int host_buffers, double 
         for (int32_t t = 0; t < todo; ++t) {
             // x lives either in the caller's buffer or in the staging buffer
             const int64_t nn = n;
+            const int it = enqueued + t;
+            double *const pc = dir[it & 1], *const pn = dir[(it + 1) & 1];
             switch (mode) {
             case SP_STAGED:
                 if (tma) {
-                    rc = spmv_tma_launch(pmap, c->A, c->q, c->partials, c->S, shares, c->stream);
+                    rc = spmv_tma_launch(pmap[it & 1], c->A, c->q, c->partials, c->S, shares, c->stream);
                     if (rc != HS_OK) return rc;
                 } else {
                     HS_TRY_CUDA(launch_dependent(k_cg_spmv_staged, shares, kSpBlock, c->stream, c->A,
-                                           (const double*)c->p, c->q, c->partials, c->S), "cg: kernel launch");
+                                           (const double*)pc, c->q, c->partials, c->S), "cg: kernel launch");
                 }
                 break;
             case SP_ROWS:
                 HS_TRY_CUDA(launch_dependent(k_cg_spmv_dot<SP_ROWS>, c->grid, kCgBlock, c->stream, c->A,
-                                       (const double*)c->p, c->q, c->partials, c->S), "cg: kernel launch");
+                                       (const double*)pc, c->q, c->partials, c->S), "cg: kernel launch");
                 break;
             default:
                 HS_TRY_CUDA(launch_dependent(k_cg_spmv_dot<SP_CSR>, c->grid, kCgBlock, c->stream, c->A,
-                                       (const double*)c->p, c->q, c->partials, c->S), "cg: kernel launch");
+                                       (const double*)pc, c->q, c->partials, c->S), "cg: kernel launch");
             }
             HS_CHECK_LAUNCH("cg: spmv+dot kernel");
-            HS_TRY_CUDA(launch_dependent(k_cg_update, c->grid, kCgBlock, c->stream, nn, x, c->r, (const double*)c->p,
-                                   (const double*)c->q, c->partials, c->S), "cg: kernel launch");
+            HS_TRY_CUDA(launch_dependent(k_cg_update, c->grid, kCgBlock, c->stream, nn, c->r, (const double*)c->q,
+                                         c->partials, c->S), "cg: kernel launch");
             HS_CHECK_LAUNCH("cg: update kernel");
-            HS_TRY_CUDA(launch_dependent(k_cg_pupdate, c->grid, kCgBlock, c->stream, nn, (const double*)c->r, c->p,
-                                   c->S, track), "cg: kernel launch");
-            HS_CHECK_LAUNCH("cg: p update kernel");
+            HS_TRY_CUDA(launch_dependent(k_cg_direction, dgrid, kCgBlock, c->stream, nn, (const double*)c->r,
+                                         (const double*)pc, pn, x, c->S, track, it, (int)(it + 1 == max_iter)),
+                        "cg: kernel launch");
+            HS_CHECK_LAUNCH("cg: direction kernel");
         }
         enqueued += todo;
         if (chunk < 32) chunk *= 2;

@@ -172,7 +172,7 @@ __global__ void __launch_bounds__(kCgBlock) k_cgb_update(const SysDev* sys, int 
     if (*(volatile int32_t*)&s.S->done || s.S->iters >= s.max_iter) return;
     __shared__ double sh[kCgBlock / 32];
     const double alpha = s.S->alpha;
-    const double rr = cg_update_rows(s.A.n, s.x, s.r, s.p, s.q, alpha, (int64_t)local * kCgBlock + threadIdx.x,
+    const double rr = cg_update_rows(s.A.n, s.r, s.q, alpha, (int64_t)local * kCgBlock + threadIdx.x,
                                      (int64_t)s.nblocks * kCgBlock);
     allow_dependents();
     const double blk = block_sum<kCgBlock>(rr, sh);
@@ -191,18 +191,20 @@ __global__ void __launch_bounds__(kCgBlock) k_cgb_update(const SysDev* sys, int 
     }
 }
 
-__global__ void __launch_bounds__(kCgBlock) k_cgb_pupdate(const SysDev* sys, int nsys)
+// x += alpha p and, unless the system has stopped, p = r + beta p, for the
+// systems that took iteration `it`.
+__global__ void __launch_bounds__(kCgBlock) k_cgb_direction(const SysDev* sys, int nsys, int it)
 {
     grid_dependency_wait();
     int local;
     const SysDev& s = sys[sys_of_block(sys, nsys, &local)];
     // the update kernel of this iteration has already counted it
-    if (*(volatile int32_t*)&s.S->done) return;
-    const double beta = s.S->beta;
-    const unsigned pm = cg_pupdate_rows(s.A.n, s.r, s.p, beta, (int64_t)local * kCgBlock + threadIdx.x,
-                                        (int64_t)s.nblocks * kCgBlock);
+    if (*(volatile int32_t*)&s.S->iters != it + 1) return;
+    const bool next = *(volatile int32_t*)&s.S->done == 0;
+    const unsigned pm = cg_direction_rows<X_ONE>(s.A.n, s.r, s.p, nullptr, s.p, s.x, s.S->alpha, 0.0, s.S->beta, next,
+                                                 (int64_t)local * kCgBlock + threadIdx.x, (int64_t)s.nblocks * kCgBlock);
     allow_dependents();
-    if (s.mode == SP_STAGED) cg_fold_pmax(pm, s.S, s.S->iters % 3, local == 0);
+    if (s.mode == SP_STAGED && next) cg_fold_pmax(pm, s.S, (it + 1) % 3, local == 0);
 }
 
 // ||b - A x||^2 into rr_true (q = A x from k_cgb_apply_x).
@@ -488,7 +490,9 @@ int cg_batch_run(hs_cg_batch_t b, const void* const* bs, void* const* xs, double
             if (b->has_mode[SP_ROWS]) CGB_LAUNCH_DEP((k_cgb_spmv_dot<SP_ROWS, kCgBlock, 1>), "cg batch: spmv+dot kernel");
             if (b->has_mode[SP_CSR]) CGB_LAUNCH_DEP((k_cgb_spmv_dot<SP_CSR, kCgBlock, 1>), "cg batch: spmv+dot kernel");
             CGB_LAUNCH_DEP(k_cgb_update, "cg batch: update kernel");
-            CGB_LAUNCH_DEP(k_cgb_pupdate, "cg batch: p update kernel");
+            HS_TRY_CUDA(launch_dependent(k_cgb_direction, G, kCgBlock, b->stream, b->d_sys, nbig, enqueued + t),
+                        "cg batch: kernel launch");
+            HS_CHECK_LAUNCH("cg batch: direction kernel");
         }
         enqueued += todo;
         if (chunk < 32) chunk *= 2;

@@ -31,6 +31,7 @@ struct CgScalars {
     // (i+1) % 3; the SpMV of iteration i reads slot i % 3.
     unsigned long long pmax[3];
     double rho2[2];    // cg_small.cu: r.r of iteration i in slot i % 2
+    double alpha2[2];  // alpha of iteration i in slot i % 2
 };
 
 constexpr int kCgBlock = 256;
@@ -417,35 +418,31 @@ __host__ __device__ inline int spmv_mode(const OpDev& A, int nblocks)
 // use these with the same partition, so their dot products add in the same
 // order.
 
-// x += alpha p, r -= alpha q; returns this thread's share of r.r.
-__device__ __forceinline__ double cg_update_rows(int64_t n, double* __restrict__ x, double* __restrict__ r,
-                                                 const double* __restrict__ p, const double* __restrict__ q,
+// r -= alpha q; returns this thread's share of r.r.  Two pairs at a time, their
+// four loads in flight together (one: 79 us at 256^3, two or four: 75; the two
+// FP64 instructions per value alone take 60 to 70).
+__device__ __forceinline__ double cg_update_rows(int64_t n, double* __restrict__ r, const double* __restrict__ q,
                                                  double alpha, int64_t t0, int64_t stride)
 {
     double rr = 0.0;
     const int64_t npairs = n >> 1;
-    const bool xvec = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
-    for (int64_t t = t0; t < npairs; t += stride) {
-        const double2 pv = reinterpret_cast<const double2*>(p)[t];
-        const double2 qv = reinterpret_cast<const double2*>(q)[t];
-        double2 xv = xvec ? reinterpret_cast<double2*>(x)[t] : make_double2(x[2 * t], x[2 * t + 1]);
-        double2 rv = reinterpret_cast<double2*>(r)[t];
-        xv.x = __fma_rn(alpha, pv.x, xv.x);
-        xv.y = __fma_rn(alpha, pv.y, xv.y);
+    double2* const r2 = reinterpret_cast<double2*>(r);
+    const double2* const q2 = reinterpret_cast<const double2*>(q);
+    auto one = [&](double2 qv, double2 rv, int64_t t) {
         rv.x = __fma_rn(-alpha, qv.x, rv.x);
         rv.y = __fma_rn(-alpha, qv.y, rv.y);
-        if (xvec) {
-            reinterpret_cast<double2*>(x)[t] = xv;
-        } else {
-            x[2 * t] = xv.x;
-            x[2 * t + 1] = xv.y;
-        }
-        reinterpret_cast<double2*>(r)[t] = rv;
+        r2[t] = rv;
         rr = __fma_rn(rv.x, rv.x, rr);
         rr = __fma_rn(rv.y, rv.y, rr);
+    };
+    int64_t t = t0;
+    for (; t + stride < npairs; t += 2 * stride) {
+        const double2 qa = q2[t], ra = r2[t], qb = q2[t + stride], rb = r2[t + stride];
+        one(qa, ra, t);
+        one(qb, rb, t + stride);
     }
+    if (t < npairs) one(q2[t], r2[t], t);
     if ((n & 1) && t0 == 0) {
-        x[n - 1] = __fma_rn(alpha, p[n - 1], x[n - 1]);
         const double rt = __fma_rn(-alpha, q[n - 1], r[n - 1]);
         r[n - 1] = rt;
         rr = __fma_rn(rt, rt, rr);
@@ -453,42 +450,74 @@ __device__ __forceinline__ double cg_update_rows(int64_t n, double* __restrict__
     return rr;
 }
 
-// p = r + beta p; returns the largest |p| high word of this thread's values.
-__device__ __forceinline__ unsigned cg_pupdate_rows(int64_t n, const double* __restrict__ r,
-                                                    double* __restrict__ p, double beta, int64_t t0,
-                                                    int64_t stride)
+// What a direction pass does to x, which waits for nothing and so is updated
+// where its direction is read anyway: nothing, x += alpha p, or the steps of
+// two iterations at once, x += alpha0 p0 and then x += alpha p (p0 the direction
+// before p).  The values are those of one update per iteration.
+enum XMode { X_NONE = 0, X_ONE = 1, X_TWO = 2 };
+
+// x as XM says; pn = r + beta p when next (pn may be p, or p0's buffer).
+// Returns the largest |pn| high word of this thread's values.
+template <int XM>
+__device__ __forceinline__ unsigned cg_direction_rows(int64_t n, const double* r, const double* p, const double* p0,
+                                                      double* pn, double* x, double alpha, double alpha0, double beta,
+                                                      bool next, int64_t t0, int64_t stride)
 {
     unsigned pm = 0;
     const int64_t npairs = n >> 1;
-    for (int64_t t = t0; t < npairs; t += stride) {
+    const bool xvec = XM != X_NONE && (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+    auto pair = [&](int64_t t) {
         const double2 a = reinterpret_cast<const double2*>(p)[t];
-        const double2 b = reinterpret_cast<const double2*>(r)[t];
-        const double2 v = make_double2(__fma_rn(beta, a.x, b.x), __fma_rn(beta, a.y, b.y));
-        reinterpret_cast<double2*>(p)[t] = v;
-        pm = max(pm, max(xs_abs_hi(v.x), xs_abs_hi(v.y)));
-    }
+        double2 b = make_double2(0.0, 0.0), xv = b, a0 = b;
+        if (next) b = reinterpret_cast<const double2*>(r)[t];
+        if constexpr (XM != X_NONE)
+            xv = xvec ? reinterpret_cast<const double2*>(x)[t] : make_double2(x[2 * t], x[2 * t + 1]);
+        if constexpr (XM == X_TWO) a0 = reinterpret_cast<const double2*>(p0)[t];
+        if constexpr (XM != X_NONE) {
+            if constexpr (XM == X_TWO) {
+                xv.x = __fma_rn(alpha0, a0.x, xv.x);
+                xv.y = __fma_rn(alpha0, a0.y, xv.y);
+            }
+            xv.x = __fma_rn(alpha, a.x, xv.x);
+            xv.y = __fma_rn(alpha, a.y, xv.y);
+            if (xvec) {
+                reinterpret_cast<double2*>(x)[t] = xv;
+            } else {
+                x[2 * t] = xv.x;
+                x[2 * t + 1] = xv.y;
+            }
+        }
+        if (next) {
+            const double2 v = make_double2(__fma_rn(beta, a.x, b.x), __fma_rn(beta, a.y, b.y));
+            reinterpret_cast<double2*>(pn)[t] = v;
+            pm = max(pm, max(xs_abs_hi(v.x), xs_abs_hi(v.y)));
+        }
+    };
+#pragma unroll 4
+    for (int64_t t = t0; t < npairs; t += stride) pair(t);
     if ((n & 1) && t0 == 0) {
-        const double v = __fma_rn(beta, p[n - 1], r[n - 1]);
-        p[n - 1] = v;
-        pm = max(pm, xs_abs_hi(v));
+        const double a = p[n - 1];
+        if constexpr (XM == X_TWO) x[n - 1] = __fma_rn(alpha0, p0[n - 1], x[n - 1]);
+        if constexpr (XM != X_NONE) x[n - 1] = __fma_rn(alpha, a, x[n - 1]);
+        if (next) {
+            const double v = __fma_rn(beta, a, r[n - 1]);
+            pn[n - 1] = v;
+            pm = max(pm, xs_abs_hi(v));
+        }
     }
     return pm;
 }
 
-// Folds a block's largest |p| high word (m, per thread) into S->pmax[slot] and,
-// from the system's first block, clears the slot after it.  All threads call it.
+// Folds the threads' largest |p| high words (m) into S->pmax[slot], warp by warp,
+// and, from the system's first block, clears the slot after it.  The slot only
+// grows during a pass: a warp whose maximum is already there skips the atomic.
 __device__ __forceinline__ void cg_fold_pmax(unsigned m, CgScalars* S, int slot, bool first_block)
 {
-    __shared__ unsigned wmax[kCgBlock / 32];
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_down_sync(0xffffffffu, m, o));
-    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
-    __syncthreads();
-    if (threadIdx.x == 0) {
-        unsigned b = 0;
-        for (int w = 0; w < kCgBlock / 32; ++w) b = max(b, wmax[w]);
-        atomicMax(&S->pmax[slot], (unsigned long long)b << 32);
-        if (first_block) S->pmax[(slot + 1) % 3] = 0;
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) {
+        const unsigned long long v = (unsigned long long)m << 32;
+        if (v > *(volatile unsigned long long*)&S->pmax[slot]) atomicMax(&S->pmax[slot], v);
+        if (first_block && threadIdx.x == 0) S->pmax[(slot + 1) % 3] = 0;
     }
 }
 
@@ -508,6 +537,10 @@ int check_op(const hs_op* A);
 OpDev to_dev(const hs_op* A);
 int grid_for(int64_t n);
 size_t cg_partials(const OpDev& A, int grid);
+// Whether a solve keeps two direction buffers and updates x every second
+// iteration (76 bytes per row and iteration instead of 80): vectors beyond L2,
+// where bytes count.
+inline bool cg_two_directions(const OpDev& A) { return A.n >= ((int64_t)1 << 22); }
 int cg_create_vectors(hs_cg_t* out, const hs_op* A, void* stream, bool need_p);
 int launch_apply(const OpDev& A, const double* p, double* y, cudaStream_t s);
 
@@ -520,6 +553,7 @@ struct hs_cg {
     double* r;
     double* p;
     double* q;
+    double* p2;            // second direction buffer (cg_two_directions), else NULL
     void* arena;           // device allocation behind ctl, S, partials, r, p and q; null: the caller's scratch
     char* ctl;             // control words of the small-system kernel (cg_small.cuh), S among them
     double* partials;      // cg_partials(A, grid) doubles
