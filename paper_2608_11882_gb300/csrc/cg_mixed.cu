@@ -43,6 +43,9 @@ struct MxScalars {
     uint32_t ticket;
     int32_t zero_rhs;
     int32_t first;        // 1 until ||b|| has been computed
+    int32_t inner;        // iterations of the current inner solve
+    int32_t pad;
+    double alpha2[2];     // alpha of its iteration i in slot i % 2
 };
 
 struct OpDev32 {
@@ -205,6 +208,7 @@ __global__ void __launch_bounds__(kCgBlock)
         if (rr_tot > 0.0 && need * need / rr_tot > f2) f2 = need * need / rr_tot;
         S->inner_stop = f2 * rho_tot;
         S->inner_done = 0;
+        S->inner = 0;
         S->beta = 0.0;   // the first direction of the inner solve is r itself
         S->outer_done = (S->zero_rhs || sqrt(rr_tot) / S->bnorm <= S->rtol) ? 1 : 0;
         if (S->outer_done || rho_tot == 0.0) S->inner_done = 1;
@@ -482,7 +486,10 @@ __global__ void __launch_bounds__(kCgBlock)
         if (!(tot > 0.0))
             S->inner_done = 2;
         else
+        {
             S->alpha = S->rho / tot;
+            S->alpha2[S->inner & 1] = S->alpha;
+        }
     }
 }
 
@@ -539,6 +546,61 @@ __global__ void __launch_bounds__(kCgBlock)
     }
 }
 
+// The update pass beside the SpMV that keeps both directions: r -= alpha q fused
+// with r.r, and d for two iterations at once in every second one (ODD: d +=
+// alpha0 p0, then d += alpha p, p0 the direction before p), so d is read and
+// written every second iteration: 20 bytes per row on average instead of 24.
+// What the last, even iteration of an inner solve leaves is added by
+// k_mx_correct.  r's values and the sum's order are k_mx_update's.
+template <bool ODD>
+__global__ void __launch_bounds__(kCgBlock)
+    k_mx_update_pair(int64_t n, float* __restrict__ d, float* __restrict__ r, const float* __restrict__ p,
+                     const float* __restrict__ p0, const float* __restrict__ q, double* partials, MxScalars* S)
+{
+    grid_dependency_wait();
+    if (*(volatile int32_t*)&S->inner_done) return;
+    __shared__ double sh[kCgBlock / 32];
+    const float alpha = (float)S->alpha, alpha0 = ODD ? (float)S->alpha2[0] : 0.0f;
+    Acc32 rr;
+    // the vectors hold a multiple of four values and start aligned (nx % 4 == 0)
+    const int64_t t0 = (int64_t)blockIdx.x * kCgBlock + threadIdx.x, stride = (int64_t)gridDim.x * kCgBlock;
+    const int64_t n4 = n >> 2;
+    for (int64_t t = t0; t < n4; t += stride) {
+        const float4 qv = reinterpret_cast<const float4*>(q)[t];
+        float4 rv = reinterpret_cast<float4*>(r)[t];
+        if constexpr (ODD) {
+            const float4 a = reinterpret_cast<const float4*>(p0)[t], c = reinterpret_cast<const float4*>(p)[t];
+            float4 dv = reinterpret_cast<float4*>(d)[t];
+            dv.x = __fmaf_rn(alpha, c.x, __fmaf_rn(alpha0, a.x, dv.x));
+            dv.y = __fmaf_rn(alpha, c.y, __fmaf_rn(alpha0, a.y, dv.y));
+            dv.z = __fmaf_rn(alpha, c.z, __fmaf_rn(alpha0, a.z, dv.z));
+            dv.w = __fmaf_rn(alpha, c.w, __fmaf_rn(alpha0, a.w, dv.w));
+            reinterpret_cast<float4*>(d)[t] = dv;
+        }
+        rv.x = __fmaf_rn(-alpha, qv.x, rv.x);
+        rv.y = __fmaf_rn(-alpha, qv.y, rv.y);
+        rv.z = __fmaf_rn(-alpha, qv.z, rv.z);
+        rv.w = __fmaf_rn(-alpha, qv.w, rv.w);
+        reinterpret_cast<float4*>(r)[t] = rv;
+        rr.add4(rv.x, rv.x, rv.y, rv.y, rv.z, rv.z, rv.w, rv.w);
+    }
+    allow_dependents();
+    const double blk = block_sum<kCgBlock>(rr.total(), sh);
+    if (!arrive_last(blk, partials, &S->ticket)) return;
+    const double rho_new = sum_partials(partials, gridDim.x, sh);
+    if (threadIdx.x == 0) {
+        S->ticket = 0;
+        S->iters += 1;
+        S->inner += 1;
+        if (rho_new <= S->inner_stop) {
+            S->inner_done = 1;
+        } else {
+            S->beta = rho_new / S->rho;
+        }
+        S->rho = rho_new;
+    }
+}
+
 __global__ void __launch_bounds__(kCgBlock)
     k_mx_pupdate(int64_t n, const float* __restrict__ r, float* __restrict__ p, MxScalars* S)
 {
@@ -560,13 +622,17 @@ __global__ void __launch_bounds__(kCgBlock)
         for (int64_t t = n4 << 2; t < n; ++t) p[t] = __fmaf_rn(beta, p[t], r[t]);
 }
 
-// x += d in FP64.
+// x += d in FP64; first d gets what an inner solve of an odd number of
+// iterations left (p: its last direction; nullptr: d is complete).
 __global__ void __launch_bounds__(kCgBlock)
-    k_mx_correct(int64_t n, double* __restrict__ x, const float* __restrict__ d)
+    k_mx_correct(int64_t n, double* __restrict__ x, const float* __restrict__ d, const float* __restrict__ p,
+                 const MxScalars* S)
 {
+    const bool left = p != nullptr && (S->inner & 1) != 0;
+    const float alpha = (float)S->alpha2[0];
     for (int64_t t = (int64_t)blockIdx.x * kCgBlock + threadIdx.x; t < n;
          t += (int64_t)gridDim.x * kCgBlock)
-        x[t] += (double)d[t];
+        x[t] += (double)(left ? __fmaf_rn(alpha, p[t], d[t]) : d[t]);
 }
 
 void cg_mixed_release(CgMixed* m, cudaStream_t s)
@@ -632,7 +698,8 @@ int cg_run_mixed(hs_cg* c, const void* b_in, void* x_inout, int host_buffers, do
             break;
         }
         if (m->S_host->iters >= max_iter) break;
-        // inner FP32 solve
+        // inner FP32 solve; with tma its direction i is in the buffer this one names for even i
+        const float* const even = m->tma ? (m->pcur ? m->p : m->p2) : nullptr;
         int32_t inner = 0;
         int chunk = 4;
         for (;;) {
@@ -652,8 +719,10 @@ int cg_run_mixed(hs_cg* c, const void* b_in, void* x_inout, int host_buffers, do
                                                  m->pmaps[m->pcur], m->A32, pn, m->q, m->partials, m->S),
                                 "cg mixed: kernel launch");
                     HS_CHECK_LAUNCH("cg mixed: p update + spmv + dot kernel");
-                    HS_TRY_CUDA(launch_dependent(k_mx_update, G, kCgBlock, c->stream, n, m->d, m->r,
-                                                 (const float*)pn, (const float*)m->q, m->partials, m->S),
+                    const float* po = m->pcur ? m->p2 : m->p;
+                    HS_TRY_CUDA(launch_dependent((inner + t) & 1 ? k_mx_update_pair<true> : k_mx_update_pair<false>, G,
+                                                 kCgBlock, c->stream, n, m->d, m->r, (const float*)pn, po,
+                                                 (const float*)m->q, m->partials, m->S),
                                 "cg mixed: kernel launch");
                     HS_CHECK_LAUNCH("cg mixed: update kernel");
                     m->pcur ^= 1;
@@ -694,7 +763,7 @@ int cg_run_mixed(hs_cg* c, const void* b_in, void* x_inout, int host_buffers, do
         if (m->S_host->inner_done == 4)
             return fail(HS_ECUDA, "cg_run: a bounded wait in the TMA-staged FP32 SpMV ran out and its loads "
                                   "in flight did not complete in time; treat the CUDA context as suspect");
-        k_mx_correct<<<G, kCgBlock, 0, c->stream>>>(n, x, m->d);   // x += d (FP64)
+        k_mx_correct<<<G, kCgBlock, 0, c->stream>>>(n, x, m->d, even, m->S);   // x += d (FP64)
         HS_CHECK_LAUNCH("cg mixed: correction kernel");
         ++outer;
     }
