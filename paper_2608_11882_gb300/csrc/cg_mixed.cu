@@ -17,6 +17,7 @@
 // and the residual norms are FP64 device scalars.  Refinement converges while
 // kappa(A) times FP32's unit roundoff is well below one (about 6e-3 for the
 // 512^3 Laplacian).
+#include <algorithm>
 #include <cmath>
 #include <cstring>
 #include <new>
@@ -312,6 +313,9 @@ __global__ void __launch_bounds__(kCgBlock)
 // per SpMV and 141.8-142.9 ms per solve (one wave of equal shares was slower
 // there: 144.1-144.5 ms); folded, with 1216 blocks of fixed 14-plane items (1.6
 // waves), 52.8 us per launch and 132.6-132.7 ms; folded, one wave: 131.0 ms.
+// Without a lower bound of blocks per SM the compiler held the kernel to 44
+// registers and the solve's iteration took 139 us at 256^3 and 544 at 400^3; with
+// it 56 registers, four resident blocks instead of five, 127 and 445 us.
 constexpr int kMxTW = 128, kMxTY = 8, kMxD = 4, kMxBW = 136, kMxNst = 4;
 constexpr uint32_t kMxBoxBytes = (kMxTY + 2) * kMxBW * sizeof(float);
 constexpr int kMxStage = (int)((kMxBoxBytes + 127) / 128 * 128 / sizeof(float));
@@ -319,7 +323,7 @@ static_assert(kMxBW * sizeof(float) % 16 == 0 && kMxD * sizeof(float) == 16, "TM
 static_assert(kMxTY * 32 == kCgBlock, "one warp per tile row");
 static_assert(2 * kMxTY <= 32, "one warp forms the halo columns");
 
-__global__ void __launch_bounds__(kCgBlock)
+__global__ void __launch_bounds__(kCgBlock, 1)
     k_mx_spmv_tma(const __grid_constant__ CUtensorMap rmap, const __grid_constant__ CUtensorMap pmap,
                   OpDev32 A, float* __restrict__ pn, float* __restrict__ q, double* partials, MxScalars* S)
 {
@@ -551,7 +555,9 @@ __global__ void __launch_bounds__(kCgBlock)
 // alpha0 p0, then d += alpha p, p0 the direction before p), so d is read and
 // written every second iteration: 20 bytes per row on average instead of 24.
 // What the last, even iteration of an inner solve leaves is added by
-// k_mx_correct.  r's values and the sum's order are k_mx_update's.
+// k_mx_correct.  Four blocks per SM with the loop unrolled by four: 127.3 us per
+// iteration at 256^3 and 445 at 400^3, against 130.7 and 511 with eight (and the
+// update that took d every time: 138.9 and 544).
 template <bool ODD>
 __global__ void __launch_bounds__(kCgBlock)
     k_mx_update_pair(int64_t n, float* __restrict__ d, float* __restrict__ r, const float* __restrict__ p,
@@ -565,6 +571,7 @@ __global__ void __launch_bounds__(kCgBlock)
     // the vectors hold a multiple of four values and start aligned (nx % 4 == 0)
     const int64_t t0 = (int64_t)blockIdx.x * kCgBlock + threadIdx.x, stride = (int64_t)gridDim.x * kCgBlock;
     const int64_t n4 = n >> 2;
+#pragma unroll 4
     for (int64_t t = t0; t < n4; t += stride) {
         const float4 qv = reinterpret_cast<const float4*>(q)[t];
         float4 rv = reinterpret_cast<float4*>(r)[t];
@@ -720,7 +727,7 @@ int cg_run_mixed(hs_cg* c, const void* b_in, void* x_inout, int host_buffers, do
                                 "cg mixed: kernel launch");
                     HS_CHECK_LAUNCH("cg mixed: p update + spmv + dot kernel");
                     const float* po = m->pcur ? m->p2 : m->p;
-                    HS_TRY_CUDA(launch_dependent((inner + t) & 1 ? k_mx_update_pair<true> : k_mx_update_pair<false>, G,
+                    HS_TRY_CUDA(launch_dependent((inner + t) & 1 ? k_mx_update_pair<true> : k_mx_update_pair<false>, std::min(G, kNumSMs * 4),
                                                  kCgBlock, c->stream, n, m->d, m->r, (const float*)pn, po,
                                                  (const float*)m->q, m->partials, m->S),
                                 "cg mixed: kernel launch");
