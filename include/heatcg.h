@@ -268,7 +268,7 @@ int heat_batch_create(hs_batch_t* out, const hs_heat_t* grids, const int64_t* st
 
 /* heat_batch_create with the work split chosen per grid.  kz[i] >= 1 splits
  * each step of grid i into z-chunks of kz[i] planes (each chunk of each column
- * tile is one item); 0 leaves it to the library (chunks of 32 planes).
+ * tile is one item); 0 leaves it to the library (equal chunks of up to 32 planes).
  * tile_w[i] is the column tile width: 64 (64 x 8 columns for FP64 grids,
  * 64 x 16 for FP32), 32 (32 x 16, FP32 32 x 32) or 0 for the
  * library's choice (the one that stages fewer values per plane, so narrow

@@ -320,7 +320,9 @@ __device__ __forceinline__ bool batch_dispatch(const BatchGrid& G, const CUtenso
     return batch_item<float, K_F32, TW>(G, map, m, t, ring, bars, seq, mx, err);
 }
 
-__global__ void __launch_bounds__(32 * kBatchTY, 8) k_heat_batch(BatchDev B)
+// Seven blocks per SM at 72 registers: 32.2 ms for 256 uneven grids, against 35.9
+// with eight at 64, which spill, 32.4 with six and 34.4 with five.
+__global__ void __launch_bounds__(32 * kBatchTY, 7) k_heat_batch(BatchDev B)
 {
     __shared__ __align__(128) long long ring[kBatchNst * kBatchSlot];
     __shared__ __align__(8) uint64_t bars[kBatchNst];
@@ -380,14 +382,16 @@ using namespace hcg;
 
 namespace {
 
-// Planes per work item when the caller leaves it to the library: chunks of 32
-// planes.  A grid's step may start only when its previous step is complete,
-// so the time one item takes bounds how fast a grid's chain of steps can go;
-// 32-plane chunks measured fastest on the 256-grid workload (ahead of whole
-// columns by 1.5x and of 16-plane chunks).
+// Planes per work item when the caller leaves it to the library: as few equal
+// chunks as keep to 32 planes.  A grid's step may start only when its previous
+// step is complete, so the time one item takes bounds how fast a grid's chain of
+// steps can go, and a grid of 33 planes in chunks of 32 and 1 waits for the long
+// one.  256 uneven grids: 31.4 ms, with 32-plane chunks and a remainder 32.2;
+// equal chunks of up to 24 31.9, 36 32.7, 48 36.9.
 int batch_default_kz(const HeatGeom& g, int)
 {
-    return g.nz < 32 ? g.nz : 32;
+    const int chunks = (g.nz + 31) / 32;
+    return (g.nz + chunks - 1) / chunks;
 }
 
 // Tile width when the caller leaves it to the library: the one that stages
