@@ -576,7 +576,8 @@ __global__ void __launch_bounds__(kNT, 3)
 // for the neighbours.  The brick partials and their order are k_cg_small's, so
 // the result is the same bit for bit.  Bound by latency: three barriers, two
 // sums over the partials and the loads of p's halo per iteration.
-__global__ void __launch_bounds__(kNT, 2) k_cg_one(const CgSmallSys* __restrict__ sys, unsigned long long* bar, int* err)
+template <int MINB>
+__global__ void __launch_bounds__(kNT, MINB) k_cg_one(const CgSmallSys* __restrict__ sys, unsigned long long* bar, int* err)
 {
     __shared__ __align__(16) long long sm[kKZ * kPlane];
     __shared__ double red[2][kNT];
@@ -780,14 +781,18 @@ int cg_small_launch(const CgSmallSys* sys, const CgSmallGroup* groups, int ngrou
                     unsigned long long* bar, int* err, cudaStream_t stream)
 {
     // asked once per process (a single GPU)
-    static const int slots = resident_blocks(k_cg_small), slots_one = resident_blocks(k_cg_one);
+    static const int slots = resident_blocks(k_cg_small), slots_one = resident_blocks(k_cg_one<2>),
+                     slots_sm = resident_blocks(k_cg_one<1>);
     if (slots < 1) return fail(HS_ECUDA, "cg: no resident block of the small-system kernel");
+    // a block per brick in registers: one per SM with all the registers it likes
+    // (64^3 11.25 us per iteration), or two (11.73; 80^3 15.5 against 18.9 in k_cg_small)
     const bool one = single && bricks <= slots_one;
-    const int blocks = (int)std::min<int64_t>(bricks, slots);   // all bricks where one holds
+    const void* kern = !one ? (const void*)k_cg_small
+                       : bricks <= slots_sm ? (const void*)k_cg_one<1> : (const void*)k_cg_one<2>;
+    const int blocks = one ? (int)bricks : (int)std::min<int64_t>(bricks, slots);
     void* args_one[] = {(void*)&sys, (void*)&bar, (void*)&err};
     void* args[] = {(void*)&sys, (void*)&groups, (void*)&ngroups, (void*)&bar, (void*)&err};
-    const cudaError_t e = cudaLaunchCooperativeKernel(one ? (const void*)k_cg_one : (const void*)k_cg_small,
-                                                      dim3((unsigned)blocks), dim3(kNT), one ? args_one : args, 0,
+    const cudaError_t e = cudaLaunchCooperativeKernel(kern, dim3((unsigned)blocks), dim3(kNT), one ? args_one : args, 0,
                                                       stream);
     if (e != cudaSuccess) {
         (void)cudaGetLastError();

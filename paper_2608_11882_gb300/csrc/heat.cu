@@ -665,10 +665,10 @@ int pick_kc_stream(const HeatGeom& g, int arith)
 // Whether heat_step advances this handle with the multi-step kernel: grids
 // below 2^22 points, 2^23 in FP32, unless the caller asked for another schedule
 // or depth.  Measured per step, Interior + Boundary launches (FP32: the blocked
-// pass) against it: 64^3 FP64 14.4 / 3.8 us, FP32 9.3 / 2.6; 128^3 FP64 18.5 /
-// 13.5, FP32 10.3 / 5.9; 160^3 FP64 27.6 / 25.5, FIXED64 24.8 / 20.0, FP32 13.4
-// / 7.9; 192^3 FP64 32.8 / 35.6, FIXED64 28.8 / 29.1, FP32 13.4 / 10.8; 224^3
-// FP32 20.6 / 21.0.
+// pass) against it: 64^3 FP64 14.4 / 3.5 us, FP32 9.3 / 2.5; 128^3 FP64 18.5 /
+// 12.2, FP32 10.3 / 6.0; 160^3 FP64 27.5 / 23.6, FIXED64 24.7 / 19.6, FP32 13.4
+// / 8.0; 176^3 FP64 29.5 / 31.1, FIXED64 24.7 / 25.5; 192^3 FP32 13.4 / 10.7;
+// 208^3 FP32 13.4 / 15.4.
 bool use_multi(const hs_heat_desc* d, const hs_heat* h)
 {
     if (d->flags & (HS_SCHED_FULL | HS_VARKAPPA)) return false;

@@ -10,10 +10,11 @@
 // values through its own stale L1 lines), converts it once, and stores the new
 // values; all loads of a brick are in flight at once, where the streaming
 // kernel waits plane by plane.  A step of a grid with one brick per block is
-// bound by latency: load, convert, store, barrier (64^3 FP64 3.8 us, FP32 2.6);
+// bound by latency: load, convert, store, barrier (64^3 FP64 3.5 us, FP32 2.5);
 // with several, by instruction issue, the z halo converted twice per four
-// planes.  Three blocks per SM: every block resident, so that two load while
-// one computes.  The per-point arithmetic is that of the other heat kernels, so
+// planes.  At least two blocks per SM, every block resident, so that one loads
+// while the other computes (held to three the kernel took 17.7 us instead of
+// 15.4 per FP64 step of 191 x 101 x 150).  The per-point arithmetic is that of the other heat kernels, so
 // results match them bit for bit, and the whole grid -- Interior and Boundary
 // planes -- is one step's work.
 #include <algorithm>
@@ -23,7 +24,7 @@
 
 namespace hcg {
 
-constexpr int kMuNT = 256, kMuKZ = 4, kMuTW = 64, kMuMinBlocks = 3;
+constexpr int kMuNT = 256, kMuKZ = 4, kMuTW = 64, kMuMinBlocks = 2;
 
 template <typename T>
 struct MultiShape {
