@@ -649,7 +649,7 @@ int pick_kc_stream(const HeatGeom& g, int arith)
     const int ry = stream_rows_for(arith);
     const int64_t tiles = (int64_t)((g.nx + tw - 1) / tw) * ((g.ny + ry - 1) / ry);
     // about four waves of 3 blocks of 16 rows per SM; the exact-sum kernel (8 rows,
-    // 8 resident blocks of 128 threads per SM) gets 64 blocks per SM, about 8
+    // 7 resident blocks of 128 threads per SM) gets 64 blocks per SM, about 9
     // waves of 27-plane chunks at 512^3 -- measured ahead of 4 waves of longer
     // chunks and 12 waves of shorter ones
     const int64_t target = (int64_t)kNumSMs * (arith == A_F64_XS ? 16 : 3) * 4;
@@ -657,7 +657,15 @@ int pick_kc_stream(const HeatGeom& g, int arith)
     int64_t chunks = (target + tiles - 1) / tiles;
     if (chunks < 1) chunks = 1;
     int64_t kc = (planes + chunks - 1) / chunks;
-    if (kc < 8) kc = 8;
+    // every chunk stages two planes more than it writes: 8 planes at least, and
+    // in the exact-sum kernel up to 16 where three waves remain
+    int64_t lo = 8;
+    if (arith == A_F64_XS) {
+        const int64_t wave = (int64_t)kNumSMs * 7;
+        lo = planes * tiles / (3 * wave);
+        lo = lo < 8 ? 8 : (lo > 16 ? 16 : lo);
+    }
+    if (kc < lo) kc = lo;
     if (kc > planes) kc = planes;
     return (int)kc;
 }

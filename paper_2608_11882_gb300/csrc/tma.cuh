@@ -70,6 +70,12 @@ __device__ __forceinline__ bool mbar_wait_bounded(uint64_t* bar, uint32_t parity
     return mbar_wait_until(bar, parity, clock64(), kWaitCycles);
 }
 
+// The same, reading the clock only once the first try has failed.
+__device__ __forceinline__ bool mbar_wait_quick(uint64_t* bar, uint32_t parity)
+{
+    return mbar_try_wait(bar, parity) || mbar_wait_until(bar, parity, clock64(), kWaitCycles);
+}
+
 // 3-D tiled TMA load of one box into shared memory, completing on bar.
 __device__ __forceinline__ void tma_load_3d(void* smem_dst, const CUtensorMap* map, int x, int y,
                                             int z, uint64_t* bar)
