@@ -594,7 +594,13 @@ def run_ours(args):
 
     # dominant kernel: the Interior kernel of the timed heat mode
     int_ms = statistics.mean(interior_ms)
-    roofline = interior_roofline(args.heat_mode, n, int_ms, hbm_gbs, peak_kind, heat.tdepth)
+    def launch_depth(h, launched):
+        """Steps per blocked launch (the library's choice takes deeper passes than
+        its depth where they are faster); 1 for the streaming kernel."""
+        return max(1, round(hsteps / launched)) if h.tdepth > 1 else 1
+
+    roofline = interior_roofline(args.heat_mode, n, int_ms, hbm_gbs, peak_kind,
+                                 launch_depth(heat, step_launches[0]))
 
     def pct(v, q):
         v = sorted(v)
@@ -694,8 +700,8 @@ def run_ours(args):
             if h.tdepth > 1:
                 ims = step_ev[0].elapsed_time(step_ev[1]) / nl
             else:
-                ims = h.interior_time()[0]
-            return ev0.elapsed_time(ev1), ims, out
+                ims, nl = h.interior_time()[0], 0
+            return ev0.elapsed_time(ev1), ims, out, launch_depth(h, nl)
 
         fields = {args.heat_mode: u_out_dev}
         side = {}
@@ -707,13 +713,13 @@ def run_ours(args):
             if spec["dtype"] == "f32":
                 src = src.float()
             h2 = make_heat(name)
-            seg_ms, ims, out = solve_once(h2, src)
+            seg_ms, ims, out, depth = solve_once(h2, src)
             side_tdepth = h2.tdepth
             h2.close()
             fields[name] = out
             side[name] = {"glups": lup_step / (seg_ms * 1e-3) / 1e9, "arith": spec["arith"],
                           "tdepth": side_tdepth,
-                          "roofline": interior_roofline(name, n, ims, hbm_gbs, peak_kind, side_tdepth)}
+                          "roofline": interior_roofline(name, n, ims, hbm_gbs, peak_kind, depth)}
             del src
         ref = fields["f64"].double()
         refmax = float(ref.abs().max())

@@ -184,7 +184,8 @@ int heat_upload(hs_heat_t h, const void* u, int src_is_device);
  * L >= 2 each pass over HBM advances L steps (temporal blocking: tiles with
  * an L-wide halo stream up the k axis, the intermediate time levels living
  * in shared memory and registers), then swaps; a remainder of n_steps is done
- * in shallower passes.  Small grids of the default arithmetics (below 2^22
+ * in shallower passes.  Where the library chose the depth (tdepth 0, HS_F32)
+ * and passes of four steps are faster, it takes those while four steps remain.  Small grids of the default arithmetics (below 2^22
  * points, 2^23 for HS_F32; HS_F64, HS_F32 or HS_FIXED64 with tdepth 0 or 1,
  * without HS_SCHED_FULL or HS_VARKAPPA, heat_time_interior off) run all n_steps
  * in one cooperative launch whose blocks meet at a barrier after every step,
@@ -229,7 +230,8 @@ int heat_read(hs_heat_t h, void* dst, int dst_is_device);
 int heat_steps_done(hs_heat_t h, int64_t* steps);
 
 /* The temporal depth the handle runs with (tdepth resolved: 1 = the Interior
- * + Boundary kernels every step, L >= 2 = L steps per pass). */
+ * + Boundary kernels every step, L >= 2 = L steps per pass, or four where the
+ * library chose the depth and that is faster). */
 int heat_get_tdepth(hs_heat_t h, int32_t* tdepth);
 
 /* Planes each block of the one-step Interior kernel takes (the k-chunk of

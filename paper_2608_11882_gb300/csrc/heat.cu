@@ -307,6 +307,7 @@ struct hs_heat {
     int64_t fxseq;     // fields produced since the last upload (FIXED64 slot = fxseq % 3)
     int kchunk;        // planes per Interior-kernel block
     int tdepth;        // steps per pass of the temporally blocked kernel (1: Interior + Boundary)
+    bool deep;         // the library chose the depth, and passes of four steps are faster here
     int kc_tb;         // k-planes per block of the temporally blocked kernel
     CUtensorMap maps[2];   // TMA maps of the two buffers (temporal blocking)
     CUtensorMap smaps[2];  // TMA maps of the two buffers (streaming Interior kernel)
@@ -614,13 +615,13 @@ int timed_interior(hs_heat* h)
     return HS_OK;
 }
 
-// Temporal depth when the descriptor leaves it to the library.  FP32 is bound
-// by HBM, and two steps per pass move half the bytes of one: at 512^3 the
-// L = 2 pass runs 880 GLUP/s against 761 for one step per pass, while depths 3
-// and 4 (one block per SM) fall below one step per pass.  FP64 and FIXED64 are
-// bound by the FP64 pipe and the integer pipes: blocking saves only bytes and
-// adds the halo's work.  The variable-coefficient problem runs one step per
-// pass.
+// Temporal depth when the descriptor leaves it to the library.  One step per
+// pass of FP32 is bound by HBM (174 us at 512^3); two steps per pass move half
+// the bytes (122 us), and where the tiles of 32-thread rows are the better
+// ones heat_step takes passes of four steps while that many remain (112 us;
+// tb_deep).  FP64 and FIXED64 are bound by the FP64 pipe and the integer pipes:
+// blocking saves only bytes and adds the halo's work.  The variable-coefficient
+// problem runs one step per pass.
 int default_tdepth(Arith a, uint32_t flags)
 {
     return (a == A_F32 && !(flags & HS_VARKAPPA)) ? 2 : 1;
@@ -631,16 +632,32 @@ int pick_kc_tb(const HeatGeom& g, int arith, int L)
     int TX = 0, TY = 0;
     tb_tile(arith, L, g.nx, &TX, &TY);
     const int64_t tiles = (int64_t)((g.nx + TX - 1) / TX) * ((g.ny + TY - 1) / TY);
-    // about six waves of two blocks per SM: 35-plane chunks at 512^3 in FP32,
-    // measured ahead of 27 (eight waves) and 52 or 64 (three or four)
-    const int64_t target = (int64_t)kNumSMs * 12;
-    int64_t chunks = (target + tiles - 1) / tiles;
-    if (chunks < 1) chunks = 1;
-    int64_t kc = (g.nz + chunks - 1) / chunks;
-    const int64_t floor_kc = 8 * L;                    // keep the z halo (2L planes) small
-    if (kc < floor_kc) kc = floor_kc;
-    if (kc > g.nz) kc = g.nz;
-    return (int)kc;
+    // Whole waves of resident blocks (two per SM at depth 2, one above), against
+    // chunks long enough that the 2 L halo planes and the ring's start (about
+    // three planes) stay cheap: the chunk length with the fewest planes in all,
+    // where that saves 5% or more of those of about 1824 blocks (without that
+    // margin FIXED64 at depth 4, 512^3, went from 571 to 616 us for a count 1%
+    // lower).  Chunks of more than 64 L planes are left out: their blocks drift
+    // apart and stop sharing halos in L2 (512^3 FP32 at depth 2: 121.9 us per
+    // step, 124.1 with 256-plane chunks).  Against the fixed count: 123.1 ->
+    // 121.9 there, 384^3 65.5 -> 56.5, depth 4 at 512^3 127.9 -> 112.3.
+    const int64_t slots = (int64_t)kNumSMs * (L == 2 ? 2 : 1);
+    auto planes = [&](int64_t kc) {
+        const int64_t blocks = tiles * ((g.nz + kc - 1) / kc);
+        return (blocks + slots - 1) / slots * (kc + 2 * L + 3);
+    };
+    const int64_t shortest = std::min<int64_t>(g.nz, 8 * L), longest = std::min<int64_t>(g.nz, 64 * L);
+    const int64_t chunks = (12 * (int64_t)kNumSMs + tiles - 1) / tiles;
+    int64_t best = std::max(shortest, (g.nz + chunks - 1) / chunks);
+    int64_t least = planes(best) * 19 / 20;
+    for (int64_t kc = longest; kc >= shortest; --kc) {
+        const int64_t p = planes(kc);
+        if (p < least) {
+            least = p;
+            best = kc;
+        }
+    }
+    return (int)best;
 }
 
 int pick_kc_stream(const HeatGeom& g, int arith)
@@ -895,6 +912,7 @@ int heat_create(hs_heat_t* out, const hs_heat_desc* desc)
     h->kchunk = pick_kchunk(h->g, desc->flags, desc->dtype);
     h->tdepth = desc->tdepth ? desc->tdepth : default_tdepth(h->arith, desc->flags);
     if (h->flags & HS_SCHED_FULL) h->tdepth = 1;
+    h->deep = desc->tdepth == 0 && h->tdepth > 1 && tb_deep(h->arith, h->g.nx);
     const size_t bytes = (size_t)h->g.total * h->elem;
     rc = check_user_buffers(desc, bytes);
     if (rc != HS_OK) {
@@ -1108,11 +1126,12 @@ int heat_step(hs_heat_t h, int64_t n_steps)
         return HS_OK;
     }
     if (h->tdepth > 1) {
-        // passes of tdepth steps, then the remainder in the largest built depths
+        // passes of the handle's depth, then the remainder in the largest built depths
+        const int top = h->deep ? 4 : h->tdepth;
         int64_t left = n_steps;
         static const int depths[] = {4, 3, 2};
         for (int L : depths) {
-            if (L > h->tdepth) continue;
+            if (L > top) continue;
             for (; left >= L; left -= L) {
                 const int rc = tb_pass(h, L);
                 if (rc != HS_OK) return rc;

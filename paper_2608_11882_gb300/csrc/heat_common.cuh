@@ -364,12 +364,9 @@ int heat_batch_view(hs_heat_t h, HeatBatchView* v);
 // Records that a batch advanced the handle by `steps` steps.
 int heat_batch_advance(hs_heat_t h, int64_t steps);
 
-// Thread rows of the temporally blocked kernel's block and rows per thread:
-// its region is kTbThreadRows kTbRowsPerThread rows high (the tile that plus
-// the halo of L rows on each side).
-constexpr int kTbThreadRows = 12;
-constexpr int kTbRowsPerThread = 2;
 // Output tile (x columns, y rows) of the temporally blocked kernel.
 void tb_tile(int arith, int L, int nx, int* tx, int* ty);
+// Whether passes of four steps are the fastest for a grid nx wide.
+bool tb_deep(int arith, int nx);
 
 }  // namespace hcg

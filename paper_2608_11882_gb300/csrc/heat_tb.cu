@@ -8,9 +8,9 @@
 // of NST shared-memory stages, several planes ahead of use, each completing on
 // its own mbarrier.  Level t (1..L) is computed one plane behind level t-1: a
 // thread keeps level t-1's values at k-1 and k in registers and receives the
-// value at k+1 from the level just computed; the x/y neighbours come from a
-// ping-pong shared plane per level (the neighbour between a thread's two rows
-// from its own registers).  Only level L reaches HBM, so a pass moves
+// value at k+1 from the level just computed; the x/y neighbours come from
+// shared planes per level, in FP32 with a warp per row the x neighbours by lane
+// shuffle (the neighbour between a thread's two rows from its own registers).  Only level L reaches HBM, so a pass moves
 // (8 or 16 bytes)/L per point-step plus the halo.  Positions outside the
 // interior and planes outside [0, nz) are the Dirichlet zeros at every level;
 // level 0 reads them from the zero boundary layer of the padded buffer or from
@@ -62,9 +62,8 @@ int encode_field_map(CUtensorMap* out, void* base, CUtensorMapDataType dt, size_
 // layout: REG + 2 rows of BW elements, the region in rows 1..REG and columns
 // A..A+RW-1, so the neighbour reads of the edge threads land in slack, never
 // outside.  W is 32 (a warp per thread row, FP32 tiles 120 columns wide) or,
-// for FP32 grids it covers with fewer warps, 34 (tiles 128 wide: a grid 2^k
-// wide is covered exactly).  With W = 34 a warp spans two thread rows; the
-// row is then padded so that the step from a row's last thread to the next
+// for FP32 grids whose width those tiles waste, 34 (tiles 128 wide).  With
+// W = 34 a warp spans two thread rows; the row is then padded so that the step from a row's last thread to the next
 // row's first (RT rows down, RW columns back) lands on the next group of
 // shared-memory banks, and 16-byte accesses stay free of bank conflicts.
 template <typename T, int L, int W>
@@ -74,8 +73,12 @@ struct TbShape {
     static constexpr int H = (L + V - 1) / V * V;
     static constexpr int RW = W * V;
     static constexpr int TX = RW - 2 * H;
-    static constexpr int RT = kTbRowsPerThread;
-    static constexpr int RR = kTbThreadRows;
+    static constexpr int RT = 2;
+    // FP32 warp rows: 16 (64 registers, two blocks of 16 warps per SM at depth 2);
+    // the halo rows weigh less than with 12: 512^3 125.0 -> 123.1 us per step,
+    // 1000^3 828 -> 767, at depth 4 143 -> 128.  Wider types, and rows of 34
+    // threads, would spill.
+    static constexpr int RR = std::is_same<T, float>::value && W == 32 ? 16 : 12;
     static constexpr int REG = RR * RT;
     static constexpr int TY = REG - 2 * L;
     static constexpr int NT = W * RR;
@@ -95,7 +98,10 @@ struct TbShape {
 };
 
 // Threads per row of the FP32 blocked kernel for a grid nx wide: 34 where its
-// 128-column tiles need fewer warps in x than the 120-column tiles of 32.
+// 128-column tiles take at least 15% fewer warps per output row than the
+// 120-column tiles of 32, which run faster per warp (lane shuffles).  Measured
+// at depth 2, 32 / 34: 256^3 (24% fewer) 22.8 / 21.6 us, 384^3 (15%) 58.5 /
+// 56.7, 512^3 (9%) 123.7 / 132.4, 640^3 (5%) 216 / 237.
 inline int tb_row_threads(int arith, int nx)
 {
     if (arith != A_F32) return 32;
@@ -103,9 +109,31 @@ inline int tb_row_threads(int arith, int nx)
     using Wd = TbShape<float, 2, 34>;
     static_assert(TbShape<float, 4, 32>::TX == N::TX && TbShape<float, 4, 34>::TX == Wd::TX,
                   "the FP32 tile width must not depend on the depth (one tensor-map box)");
-    const int64_t narrow = (int64_t)((nx + N::TX - 1) / N::TX) * N::WARPS;
-    const int64_t wide = (int64_t)((nx + Wd::TX - 1) / Wd::TX) * Wd::WARPS;
-    return wide < narrow ? 34 : 32;
+    const int64_t narrow = (int64_t)((nx + N::TX - 1) / N::TX) * N::WARPS * Wd::TY;
+    const int64_t wide = (int64_t)((nx + Wd::TX - 1) / Wd::TX) * Wd::WARPS * N::TY;
+    return 15 * wide <= 13 * narrow ? 34 : 32;
+}
+
+// A row of four FP32 points as Point<float>::update computes them, the sums
+// and fused multiply-adds two points at a time (the same roundings): 512^3
+// 134.8 -> 133.3 us per step, 1024^3 955 -> 938, depth 4 at 512^3 170.5 -> 165.1.
+__device__ __forceinline__ void f32_row_update(const float (&c)[4], float left, float right,
+                                               const float (&yl)[4], const float (&yh)[4],
+                                               const float (&zl)[4], const float (&zh)[4], float r,
+                                               float (&v)[4])
+{
+#pragma unroll
+    for (int i = 0; i < 4; i += 2) {
+        const float2 cc = make_float2(c[i], c[i + 1]);
+        const float2 sx = make_float2(__fadd_rn(i == 0 ? left : c[i == 0 ? 0 : i - 1], c[i + 1]),
+                                      __fadd_rn(c[i], i == 2 ? right : c[i == 2 ? 0 : i + 2]));
+        const float2 sy = __fadd2_rn(make_float2(yl[i], yl[i + 1]), make_float2(yh[i], yh[i + 1]));
+        const float2 sz = __fadd2_rn(make_float2(zl[i], zl[i + 1]), make_float2(zh[i], zh[i + 1]));
+        const float2 s = __fadd2_rn(__fadd2_rn(sx, sy), sz);
+        const float2 w = __ffma2_rn(make_float2(r, r), __ffma2_rn(make_float2(-6.0f, -6.0f), cc, s), cc);
+        v[i] = w.x;
+        v[i + 1] = w.y;
+    }
 }
 
 // The pass over one chunk of planes [kb, ke).  MASK = false is taken by blocks
@@ -122,6 +150,15 @@ __device__ __forceinline__ unsigned long long tb_chunk(const CUtensorMap* map, T
 {
     using S = TbShape<T, L, W>;
     constexpr int V = S::V, A = S::A, H = S::H, BW = S::BW, PLANE = S::PLANE, RT = S::RT;
+    // FP32 rows of 32 threads are one warp each: the x neighbours come by lane
+    // shuffle, not by one-element loads 16 bytes apart (four wavefronts each).
+    // The end lanes get their own values; a level so loses one column at each
+    // end of the region, which is L <= H columns wider than the tile.  333^3
+    // 47.2 -> 43.2 us per step, 480^3 107 -> 99.4.  With rows of 34 threads the
+    // lanes that start and end a warp would have to load theirs (157 us at 512^3
+    // against 133, with spills).
+    constexpr bool F32 = std::is_same<T, float>::value;
+    static_assert(L <= H, "end columns are not part of the tile");
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int tid = ty * W + tx;
     const int x0 = blockIdx.x * S::TX, y0 = blockIdx.y * S::TY;
@@ -157,16 +194,13 @@ __device__ __forceinline__ unsigned long long tb_chunk(const CUtensorMap* map, T
     unsigned long long mx = 0;
     T* out = dst + g.at(nvx > 0 ? X : 0, 0, 0);   // row 0 of plane 0; used when nvx > 0
 
-    int s_cur = 0, n_cur = 0;   // slot and use count of plane q
-    // unrolled by three, the period of the rotation zb <- zc <- up: the
-    // compiler renames the registers instead of copying them every plane
-#pragma unroll 3
-    for (int q = q0; q <= qlast; ++q) {
-        if (!mbar_wait_bounded(&bars[s_cur], (uint32_t)n_cur & 1u)) {
+    // plane q in slot s_cur of the ring; false: the march ends
+    auto step = [&](int q, int s_cur, uint32_t phase) -> bool {
+        if (!mbar_wait_quick(&bars[s_cur], phase)) {
             atomicExch(err, 1);
             *s_abort = 1;
         }
-        const int s_prev = s_cur == 0 ? NST - 1 : s_cur - 1;   // plane q-1 (junk at q = q0)
+        const int s_prev = (s_cur + NST - 1) % NST;   // plane q-1 (junk at q = q0)
         T up[RT][V];
 #pragma unroll
         for (int j = 0; j < RT; ++j) ld_vec(stage + s_cur * PLANE + own + j * BW, up[j]);
@@ -174,27 +208,37 @@ __device__ __forceinline__ unsigned long long tb_chunk(const CUtensorMap* map, T
         for (int t = 1; t <= L; ++t) {
             const int p = q - t;
             const T* src = (t == 1) ? stage + s_prev * PLANE + own
-                                    : lev + ((t - 2) * 2 + ((q - 1) & 1)) * PLANE + own;
+                                    : lev + ((t - 2) * NST + s_prev) * PLANE + own;
             T ym[V], yp[V], v[RT][V];
             ld_vec(src - BW, ym);
             ld_vec(src + RT * BW, yp);
             const bool zin = p >= 0 && p < g.nz;
 #pragma unroll
             for (int j = 0; j < RT; ++j) {
-                const T left = src[j * BW - 1], right = src[j * BW + V];
+                T left, right;
+                if constexpr (F32 && W == 32) {
+                    left = __shfl_up_sync(0xffffffffu, zc[t - 1][j][V - 1], 1);
+                    right = __shfl_down_sync(0xffffffffu, zc[t - 1][j][0], 1);
+                } else {
+                    left = src[j * BW - 1];
+                    right = src[j * BW + V];
+                }
+                const T(&c)[V] = zc[t - 1][j];
+                const T(&yl)[V] = j == 0 ? ym : zc[t - 1][j == 0 ? 0 : j - 1];
+                const T(&yh)[V] = j == RT - 1 ? yp : zc[t - 1][j == RT - 1 ? j : j + 1];
+                if constexpr (F32 && !EXACT) {
+                    f32_row_update(c, left, right, yl, yh, zb[t - 1][j], up[j], r, v[j]);
+                } else {
 #pragma unroll
-                for (int i = 0; i < V; ++i) {
-                    const T xm = i == 0 ? left : zc[t - 1][j][i - 1];
-                    const T xp = i == V - 1 ? right : zc[t - 1][j][i + 1];
-                    const T yl = j == 0 ? ym[i] : zc[t - 1][j - 1][i];
-                    const T yh = j == RT - 1 ? yp[i] : zc[t - 1][j + 1][i];
-                    const T w = Point<T, EXACT>::update(zc[t - 1][j][i], xm, xp, yl, yh, zb[t - 1][j][i],
-                                                        up[j][i], r, t == 1 ? ks : 0);
-                    // Dirichlet zeros outside the interior
-                    if constexpr (MASK)
-                        v[j][i] = (zin && in_x[i] && in_y[j]) ? w : T(0);
-                    else
-                        v[j][i] = w;
+                    for (int i = 0; i < V; ++i)
+                        v[j][i] = Point<T, EXACT>::update(c[i], i == 0 ? left : c[i - 1],
+                                                          i == V - 1 ? right : c[i + 1], yl[i], yh[i],
+                                                          zb[t - 1][j][i], up[j][i], r, t == 1 ? ks : 0);
+                }
+                if constexpr (MASK) {   // Dirichlet zeros outside the interior
+#pragma unroll
+                    for (int i = 0; i < V; ++i)
+                        if (!(zin && in_x[i] && in_y[j])) v[j][i] = T(0);
                 }
             }
 #pragma unroll
@@ -205,7 +249,7 @@ __device__ __forceinline__ unsigned long long tb_chunk(const CUtensorMap* map, T
                     zc[t - 1][j][i] = up[j][i];
                 }
             if (t < L) {
-                T* lp = lev + ((t - 1) * 2 + (q & 1)) * PLANE + own;
+                T* lp = lev + ((t - 1) * NST + s_cur) * PLANE + own;
 #pragma unroll
                 for (int j = 0; j < RT; ++j) {
                     st_vec(lp + j * BW, v[j]);
@@ -236,7 +280,7 @@ __device__ __forceinline__ unsigned long long tb_chunk(const CUtensorMap* map, T
         __syncthreads();
         if (*s_abort) {
             drain_from = q;
-            break;
+            return false;
         }
         if (tid == 0 && q > q0 && issued < qlast) {
             // plane q-1's slot is free: refill it with the next plane
@@ -246,10 +290,17 @@ __device__ __forceinline__ unsigned long long tb_chunk(const CUtensorMap* map, T
             tma_load_3d(stage + s_prev * PLANE, map, xs, ybox, pn + 1, &bars[s_prev]);
             issued = pn;
         }
-        if (++s_cur == NST) {
-            s_cur = 0;
-            ++n_cur;
-        }
+        return q < qlast;
+    };
+    // three planes per turn, the period of the ring and of the rotation zb <- zc
+    // <- up: slots are constants and registers are renamed, not copied (512^3
+    // 129.2 -> 125.0 us per step against a loop that counts its slots)
+    static_assert(NST == 3, "a turn visits each slot once");
+    uint32_t phase = 0;
+    for (int q = q0;; q += 3, phase ^= 1u) {
+        if (!step(q, 0, phase)) break;
+        if (!step(q + 1, 1, phase)) break;
+        if (!step(q + 2, 2, phase)) break;
     }
     return mx;
 }
@@ -263,8 +314,8 @@ __global__ void __launch_bounds__(TbShape<T, L, W>::NT, MINB)
     static_assert(S::TY > 0 && S::TX > 0, "tile too small for the temporal depth");
     extern __shared__ __align__(128) unsigned char smem_raw[];
     T* stage = reinterpret_cast<T*>(smem_raw);
-    T* lev = stage + NST * S::PLANE;   // level t (1..L-1), buffer b: lev + ((t-1)*2 + b) * PLANE
-    uint64_t* bars = reinterpret_cast<uint64_t*>(lev + (L - 1) * 2 * S::PLANE);
+    T* lev = stage + NST * S::PLANE;   // level t (1..L-1), slot s: lev + ((t-1) * NST + s) * PLANE
+    uint64_t* bars = reinterpret_cast<uint64_t*>(lev + (L - 1) * NST * S::PLANE);
     __shared__ int s_abort;
 
     const int tid = threadIdx.y * W + threadIdx.x;
@@ -320,7 +371,7 @@ int tb_launch_w(const TbCall& c)
     constexpr int MINB = L == 2 ? 2 : 1;
     using S = TbShape<T, L, W>;
     constexpr size_t smem =
-        sizeof(T) * (size_t)(NST + 2 * (L - 1)) * S::PLANE + NST * sizeof(uint64_t);
+        sizeof(T) * (size_t)NST * L * S::PLANE + NST * sizeof(uint64_t);
     if (c.box[0] != (uint32_t)S::BW || c.box[1] != (uint32_t)S::ROWS)
         return fail(HS_EINVAL, "heat: tensor map box %ux%u does not match the kernel's %dx%d", c.box[0],
                     c.box[1], S::BW, S::ROWS);
@@ -363,7 +414,7 @@ int tb_box(int arith, int nx, uint32_t* box_x, uint32_t* box_y)
     if (arith == A_F32) {
         const bool wide = tb_row_threads(arith, nx) == 34;
         *box_x = wide ? TbShape<float, 2, 34>::BW : TbShape<float, 2, 32>::BW;
-        *box_y = TbShape<float, 2, 32>::ROWS;
+        *box_y = wide ? TbShape<float, 2, 34>::ROWS : TbShape<float, 2, 32>::ROWS;
     } else {
         *box_x = TbShape<double, 2, 32>::BW;
         *box_y = TbShape<double, 2, 32>::ROWS;
@@ -389,6 +440,14 @@ void tb_tile(int arith, int L, int nx, int* tx, int* ty)
         tb_tile_t<float, 34>(L, tx, ty);
     else
         tb_tile_t<float, 32>(L, tx, ty);
+}
+
+// Per step, depth 2 / depth 4: 32-thread rows 220^3 15.6 / 11.8 us, 333^3 38.0 /
+// 32.9, 512^3 121.9 / 112.3, 640^3 211 / 211, 1000^3 764 / 697; 34-thread rows
+// (the depth-4 pass spills with their blocks) 256^3 21.3 / 24.1, 384^3 56.5 / 64.7.
+bool tb_deep(int arith, int nx)
+{
+    return arith == A_F32 && tb_row_threads(arith, nx) == 32;
 }
 
 int tb_launch(const TbCall& c)
