@@ -97,8 +97,9 @@ __device__ __forceinline__ bool vk_exact_ok(int emax, double b)
 // as in heat_stream.cu.
 //
 // Instruction issue (62%), the FP64 pipe (57%) and DRAM (58%) share the time, 174
-// instructions per point.  510^3: 890 us per step, 149 GLUP/s = 4.77 TB/s of the
-// 32 bytes per update; 520 x 510 x 500 1176 us.  Before: face sums in three arrays
+// instructions per point.  510^3: 856 us per step, 155 GLUP/s = 4.96 TB/s of the
+// 32 bytes per update (890 before xs_fix's shorter form, which the figures below
+// and 520 x 510 x 500's 1176 us go with).  Before: face sums in three arrays
 // (48 bytes), their products summed in 128 bits, every neighbour converted where
 // it was used, 265 instructions: 1541 us and 2400 us.  Loads through L1 instead
 // of TMA: 1178 us.  Three resident blocks either way, but held to 80 registers
