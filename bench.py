@@ -42,16 +42,15 @@ FP64_INSTR_PEAK_T = 0.625
 NOMINAL_HBM_GBS = 7900.0   # GB300 HBM3e nominal bandwidth (the measured copy rate is the roofline peak)
 # DRAM bytes per launch (dram__bytes_read.sum + dram__bytes_write.sum) of the
 # dominant kernel, from one ncu capture of the kernel as it stands, keyed by
-# (arithmetic, grid edge, steps per launch): the FP64 exact-sum Interior kernel
-# (two rows per thread, one point in four converted on the FP64 pipe) on 512^3
-# read 1187.2 MB and wrote 1025.9 MB per launch (mean of 2 launches); the FP32
-# blocked kernel at depth 2 (34-thread rows, plane loop unrolled by three) on
-# 512^3 read 626.5 MB and wrote 494.2 MB per pass (mean of 2 passes); the FIXED64
-# streaming kernel (plane loop unrolled by three) on 512^3 read 1149.5 MB and
-# wrote 1025.9 MB per launch (mean of 2 launches).
+# (arithmetic, grid edge, steps per launch), on 512^3, means of two launches: the
+# FP64 exact-sum Interior kernel (two register sets, 27-plane chunks) read 1171.6 MB
+# and wrote 1026.2 MB; the FP32 blocked kernel (120-column tiles) read 604.2 MB and
+# wrote 497.5 MB per pass of two steps, 591.1 and 495.8 MB per pass of four; the
+# FIXED64 streaming kernel (plane loop unrolled by three) read 1149.5 MB and wrote
+# 1025.9 MB.
 # Re-capture after any change to that kernel; sizes not listed report null.
-KERNEL_TRAFFIC_BYTES = {("f64", 512, 1): 2213105024, ("f32", 512, 2): 1120694016,
-                        ("fixed64", 512, 1): 2175355904}
+KERNEL_TRAFFIC_BYTES = {("f64", 512, 1): 2197791488, ("f32", 512, 2): 1101715328,
+                        ("f32", 512, 4): 1086894080, ("fixed64", 512, 1): 2175355904}
 HEAT_MODES = {
     # plain FP64 handle: FP64 fields, exact int64 neighbour sum, one FP64 FMA per point
     "f64": {"dtype": "f64", "flags": "", "arith": "f64", "bytes": 16, "bound": "hbm",

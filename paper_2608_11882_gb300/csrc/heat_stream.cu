@@ -401,13 +401,13 @@ __device__ __forceinline__ void xs_stream_body(const CUtensorMap* map, double* _
 }
 
 // kXsRows rows per tile, kXsRowsPerThread per thread, 128 threads.  Bound by
-// the integer pipe (73% busy; FP64 65%, DRAM 79% of the measured copy): the
-// planes rotate between two named sets of registers, four planes per turn of
-// the loop, so the ring's slots are constants and no register is copied, and
-// the sum of plane k's own neighbours runs before the wait for plane k + 1.
-// That takes 72 registers: seven blocks per SM instead of eight at 64, which
-// spilled.  512^3, one step: 406.5 -> 393.6 us (384.9 with xs_fix's shorter
-// form), 300^3 100.4 -> 98.4.
+// the integer and the FP64 pipe (70% and 67% busy at 320^3, 74 instructions per
+// point where the form before had 92): the planes rotate between two named sets
+// of registers, four planes per turn of the loop, so the ring's slots are
+// constants and no register is copied, and the sum of plane k's own neighbours
+// runs before the wait for plane k + 1.  That takes 72 registers: seven blocks
+// per SM instead of eight at 64.  512^3, one step: 406.5 -> 393.6 us (384.9 with
+// xs_fix's shorter form), 300^3 100.4 -> 98.4.
 template <int RY, int RT, int NST>
 __global__ void __launch_bounds__(32 * (RY / RT), 7)
     k_heat_stream_xs(const __grid_constant__ CUtensorMap map, double* __restrict__ dst, HeatGeom g,
