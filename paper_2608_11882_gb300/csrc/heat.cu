@@ -646,7 +646,9 @@ int pick_kc_tb(const HeatGeom& g, int arith, int L)
         const int64_t blocks = tiles * ((g.nz + kc - 1) / kc);
         return (blocks + slots - 1) / slots * (kc + 2 * L + 3);
     };
-    const int64_t shortest = std::min<int64_t>(g.nz, 8 * L), longest = std::min<int64_t>(g.nz, 64 * L);
+    // a launch holds 65535 chunks
+    const int64_t fit = ((int64_t)g.nz + 65534) / 65535;
+    const int64_t shortest = std::max(fit, std::min<int64_t>(g.nz, 8 * L)), longest = std::min<int64_t>(g.nz, 64 * L);
     const int64_t chunks = (12 * (int64_t)kNumSMs + tiles - 1) / tiles;
     int64_t best = std::max(shortest, (g.nz + chunks - 1) / chunks);
     int64_t least = planes(best) * 19 / 20;

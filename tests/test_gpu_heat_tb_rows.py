@@ -45,3 +45,10 @@ def test_library_choice(pkg, shape, steps):
     with pkg.Heat(shape[2], shape[1], shape[0], 0.15, dtype="f32") as h:
         assert h.tdepth == 2
     assert np.array_equal(run(pkg, u0, steps, 1), run(pkg, u0, steps, 0))
+
+
+@pytest.mark.parametrize("tdepth", [2, 4])
+def test_very_tall_grid(pkg, tdepth):
+    """More planes than 65535 chunks of the usual length hold."""
+    u0 = field((8_600_000, 1, 1))
+    assert np.array_equal(run(pkg, u0, 5, 1), run(pkg, u0, 5, tdepth))
