@@ -39,6 +39,11 @@ namespace {
 constexpr int kNT = kCgBlock, kKZ = kCgSmallKZ;
 constexpr int kPlane = 680;   // shared words per plane: 10 rows of 68 or 18 of 36 (648)
 
+// In alpha's place: A is not positive definite on p (p.q <= 0, or NaN).  alpha
+// itself is never negative; it is 0 where p.q overflows and r.r does not, and
+// the solve then goes on to max_iter, as with three launches per iteration.
+constexpr double kBreakdown = -1.0;
+
 // The thread's place in a brick of a system.
 struct Place {
     int X, Y, k0;
@@ -404,8 +409,10 @@ __global__ void __launch_bounds__(kNT, 3)
         }
         if (!sync()) return;
 
+        int most = 0;   // iterations any system of the group may take: ends the loop whatever its scalars say
+        for (int i = 0; i < nsys; ++i) most = max(most, sys[i].max_iter);
         bool relist = true;   // some system stopped: the others' bricks are shared out anew
-        for (int it = 0;; ++it) {
+        for (int it = 0; it < most; ++it) {
             if (relist) w = list(false, it);
             if (s_n == 0) break;   // the same in every block
             unsigned ended = 0;    // thread 0: a system this block keeps the scalars of stops with this iteration
@@ -433,8 +440,7 @@ __global__ void __launch_bounds__(kNT, 3)
                 const double pq = sys_sum(s.part, s.bricks, red[turn & 1]);
                 ++turn;
                 if (tid == 0) {
-                    // breakdown (A not positive definite on p): nothing more is updated
-                    s_alpha[e] = pq > 0.0 ? rho / pq : 0.0;
+                    s_alpha[e] = pq > 0.0 ? rho / pq : kBreakdown;
                     if (s_first[e] >= w.lo && !(pq > 0.0)) {
                         s.S->done = 2;
                         ended = 1;
@@ -442,6 +448,7 @@ __global__ void __launch_bounds__(kNT, 3)
                 }
                 __syncthreads();
                 const double alpha = s_alpha[e];
+                if (alpha == kBreakdown) continue;   // nothing more is updated
                 for (int g = max(w.lo, s_first[e]); g < min(w.hi, s_first[e + 1]); ++g) {
                     const int brick = g - s_first[e];
                     const Place c = place_of(s, brick, tid);
@@ -474,7 +481,7 @@ __global__ void __launch_bounds__(kNT, 3)
                 const bool xvec = (s.nx & 1) == 0 && (reinterpret_cast<uintptr_t>(s.x) & 15) == 0;
                 const int64_t sxy = (int64_t)s.pitch * s.ny, sd = (int64_t)s.nx * s.ny;
                 const double alpha = s_alpha[e];
-                if (alpha == 0.0) continue;   // breakdown: the block that keeps its scalars has ended it
+                if (alpha == kBreakdown) continue;   // the block that keeps its scalars has ended it
                 double rho = 0.0, bnorm = 0.0, rtol = 0.0;
                 if (tid == 0) {
                     rho = __ldcg(&S->rho2[it & 1]);
@@ -667,10 +674,10 @@ __global__ void __launch_bounds__(kNT, MINB) k_cg_one(const CgSmallSys* __restri
         brick_sum(pq_t, red[0], it, part_pq);
         if (!sync(false, 0u)) return;
         const double pq = sys_sum(s.part, s.bricks, red[1]);
-        if (tid == 0) s_val = pq > 0.0 ? rho / pq : 0.0;
+        if (tid == 0) s_val = pq > 0.0 ? rho / pq : kBreakdown;
         __syncthreads();
         const double alpha = s_val;
-        if (alpha == 0.0) {   // breakdown: A not positive definite on p
+        if (alpha == kBreakdown) {
             done = 2;
             break;
         }

@@ -91,3 +91,38 @@ def test_more_systems_than_one_group(pkg):
         with pkg.CG(ops[k]) as cg:
             x1, i1 = cg.run(dev(bs[k]), rtol=1e-9, max_iter=500)
         assert np.array_equal(xs[k].cpu().numpy(), x1.cpu().numpy()) and infos[k]["iters"] == i1["iters"]
+
+
+# one block per brick, several bricks per block, and fewer unknowns than either takes
+@pytest.mark.parametrize("shape", [(32, 32, 64), (33, 17, 65), (128, 128, 128), (12, 20, 18)])
+def test_overflowing_pq_ends_at_max_iter(pkg, shape):
+    """||r||^2 finite and p.q beyond the largest double: alpha is 0, x stays, and
+    the solve ends at max_iter, alone and in a batch beside a system that goes on
+    or converges.  r stays too, so p_i = (i + 1) r: the iterations are few enough
+    that no single product p[k] q[k] overflows, which would make p.q NaN."""
+    torch = require_cuda()
+    nz, ny, nx = shape
+    n = nx * ny * nz
+    b = cg_rhs(n, seed=3)
+    b /= np.linalg.norm(b)
+    p2 = b.reshape(shape)
+    its = 6
+    assert float((p2 * oracle.lap7_apply(p2)).sum()) > 4.0                     # p.q > 2.4e308
+    assert 12.0 * its ** 2 * float(np.abs(b).max()) ** 2 * 6e307 < 1.7e308     # |p[k] q[k]| of the last iteration
+    b *= np.sqrt(6e307)
+    x0 = torch.zeros(n, dtype=torch.float64, device="cuda")
+    op, other = pkg.Operator.stencil(nx, ny, nz), pkg.Operator.stencil(30, 28, 26)
+    bo = dev(cg_rhs(30 * 28 * 26, seed=1))
+    with pkg.CG(op) as cg, pkg.CG(other) as co:
+        x, info = cg.run(dev(b), x=x0.clone(), rtol=0.5, max_iter=its)
+        xo, io = co.run(bo, rtol=0.5, max_iter=its)
+    assert not info["converged"] and info["iters"] == its and torch.equal(x, x0)
+    assert abs(info["relres_recur"] - 1.0) < 1e-12 and abs(info["relres_true"] - 1.0) < 1e-12
+    assert io["converged"] and io["iters"] < its
+    for ops, bs, k in (([op, other], [dev(b), bo], 0), ([other, op], [bo, dev(b)], 1)):
+        with pkg.CGBatch(ops) as cb:
+            xs, infos = cb.run(bs, rtol=0.5, max_iter=its)
+            assert not infos[k]["converged"] and infos[k]["iters"] == its and torch.equal(xs[k], x0)
+            assert infos[1 - k]["converged"] and torch.equal(xs[1 - k], xo)
+            xs, infos = cb.run(bs, rtol=1e-8, max_iter=its)
+            assert [i["iters"] for i in infos] == [its, its] and torch.equal(xs[k], x0)
