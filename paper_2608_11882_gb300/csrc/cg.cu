@@ -109,7 +109,6 @@ __global__ void __launch_bounds__(kCgBlock)
             S->done = 2;   // breakdown: A is not positive definite on p
         } else {
             S->alpha = S->rho / tot;
-            S->alpha2[S->iters & 1] = S->alpha;
         }
     }
 }
@@ -135,28 +134,34 @@ __global__ void __launch_bounds__(kSpBlock, kSpMinBlocks)
             S->done = 2;   // breakdown: A is not positive definite on p
         } else {
             S->alpha = S->rho / tot;
-            S->alpha2[S->iters & 1] = S->alpha;
         }
     }
 }
 
-// r -= alpha q fused with r.r; the last block tests convergence
-// and forms beta.
+// r -= alpha q fused with r.r, and in a solve that stays in L2 (WITH_X) x += alpha
+// p, whose loads and stores hide behind the reduction's; the last block tests
+// convergence and forms beta.  Below 2^22 unknowns moving x to the direction pass,
+// which has no reduction, made a CSR solve slower: 48^3 3684 -> 4279 us, 33 x 47 x
+// 91 4975 -> 5955, 16 of 64^3 116 -> 128 ms.
+template <bool WITH_X>
 __global__ void __launch_bounds__(kCgBlock)
-    k_cg_update(int64_t n, double* __restrict__ r, const double* __restrict__ q, double* partials, CgScalars* S)
+    k_cg_update(int64_t n, double* __restrict__ x, double* __restrict__ r, const double* __restrict__ p,
+                const double* __restrict__ q, double* partials, CgScalars* S)
 {
     grid_dependency_wait();
     if (*(volatile int32_t*)&S->done) return;
     __shared__ double sh[kCgBlock / 32];
     const double alpha = S->alpha;
-    const double rr = cg_update_rows(n, r, q, alpha, (int64_t)blockIdx.x * kCgBlock + threadIdx.x,
-                                     (int64_t)gridDim.x * kCgBlock);
+    const int64_t t0 = (int64_t)blockIdx.x * kCgBlock + threadIdx.x, stride = (int64_t)gridDim.x * kCgBlock;
+    const double rr = WITH_X ? cg_update_xr_rows(n, x, r, p, q, alpha, t0, stride)
+                             : cg_update_rows(n, r, q, alpha, t0, stride);
     allow_dependents();
     const double blk = block_sum<kCgBlock>(rr, sh);
     if (!arrive_last(blk, partials, &S->ticket)) return;
     const double rho_new = sum_partials(partials, gridDim.x, sh);
     if (threadIdx.x == 0) {
         S->ticket = 0;
+        if (!WITH_X) S->alpha2[S->iters & 1] = alpha;   // the direction pass adds to x later
         S->iters += 1;
         S->relres = sqrt(rho_new) / S->bnorm;
         if (S->relres <= S->rtol) {
@@ -168,10 +173,27 @@ __global__ void __launch_bounds__(kCgBlock)
     }
 }
 
-// The direction pass of iteration `it`: p' = r + beta p unless the solve has
-// stopped, and x for the iterations not added to it yet -- with two direction
-// buffers (pn another buffer than p) every second iteration's, else this one's.
-// `last`: no iteration follows.  A pass enqueued past the stop does nothing.
+// p = r + beta p, for solves that update x with r.
+__global__ void __launch_bounds__(kCgBlock)
+    k_cg_pupdate(int64_t n, const double* __restrict__ r, double* __restrict__ p, CgScalars* S, int track_pmax)
+{
+    grid_dependency_wait();
+    if (*(volatile int32_t*)&S->done) return;
+    const double beta = S->beta;
+    const unsigned pm = cg_pupdate_rows(n, r, p, beta, (int64_t)blockIdx.x * kCgBlock + threadIdx.x,
+                                        (int64_t)gridDim.x * kCgBlock);
+    allow_dependents();
+    // the update kernel has counted this iteration: p is the next one's direction
+    if (track_pmax) cg_fold_pmax_block(pm, S, S->iters % 3, blockIdx.x == 0);
+}
+
+// The direction pass of iteration `it` in a large solve: p' = r + beta p unless
+// the solve has stopped, and x for the iterations not added to it yet -- with two
+// direction buffers (pn another buffer than p) every second iteration's, else
+// this one's.  `last`: no iteration follows.  A pass enqueued past the stop does
+// nothing.  256^3: 202 ms per solve, 223 with x in the update pass; a kernel for
+// each parity takes 223.5 (80 registers, fewer blocks), and one without the
+// single-buffer case 205.5.
 __global__ void __launch_bounds__(kCgBlock)
     k_cg_direction(int64_t n, const double* r, const double* p, double* pn, double* x, CgScalars* S, int track_pmax,
                    int it, int last)
@@ -442,7 +464,7 @@ int cg_create_vectors(hs_cg_t* out, const hs_op* A, void* stream, bool need_p)
     auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t s_ctl = align(sizeof(CgSmallCtl)), s_part = align(sizeof(double) * cg_partials(c->A, c->grid));
     const size_t s_vec = align(sizeof(double) * (size_t)cg_vector_len(c->A));
-    const bool two = need_p && cg_two_directions(c->A);
+    const bool two = need_p && cg_x_late(c->A);
     CG_ALLOC(c->arena, s_ctl + s_part + (two ? 4 : need_p ? 3 : 2) * s_vec);
     c->ctl = (char*)c->arena;
     c->S = &((CgSmallCtl*)c->ctl)->S;
@@ -594,6 +616,7 @@ int cg_run(hs_cg_t c, const void* b_in, void* x_inout, int host_buffers, double 
     const int track = mode == SP_STAGED;   // the staged SpMV needs p's largest exponent
     const int shares = mode == SP_STAGED ? spmv_shares(c->grid) : c->grid;
     // the staged SpMV takes p through TMA when the grid and the vectors allow
+    const bool late = cg_x_late(c->A);
     double* const dir[2] = {c->p, c->p2 ? c->p2 : c->p};   // the direction of iteration i is in dir[i % 2]
     CUtensorMap pmap[2];
     const bool tma = mode == SP_STAGED && spmv_tma_eligible(c->A, c->p, c->q, c->grid) &&
@@ -640,12 +663,18 @@ int cg_run(hs_cg_t c, const void* b_in, void* x_inout, int host_buffers, double 
                                        (const double*)pc, c->q, c->partials, c->S), "cg: kernel launch");
             }
             HS_CHECK_LAUNCH("cg: spmv+dot kernel");
-            HS_TRY_CUDA(launch_dependent(k_cg_update, c->grid, kCgBlock, c->stream, nn, c->r, (const double*)c->q,
-                                         c->partials, c->S), "cg: kernel launch");
-            HS_CHECK_LAUNCH("cg: update kernel");
-            HS_TRY_CUDA(launch_dependent(k_cg_direction, dgrid, kCgBlock, c->stream, nn, (const double*)c->r,
-                                         (const double*)pc, pn, x, c->S, track, it, (int)(it + 1 == max_iter)),
+            HS_TRY_CUDA(launch_dependent(late ? k_cg_update<false> : k_cg_update<true>, c->grid, kCgBlock, c->stream, nn,
+                                         x, c->r, (const double*)pc, (const double*)c->q, c->partials, c->S),
                         "cg: kernel launch");
+            HS_CHECK_LAUNCH("cg: update kernel");
+            if (late)
+                HS_TRY_CUDA(launch_dependent(k_cg_direction, dgrid, kCgBlock, c->stream, nn, (const double*)c->r,
+                                             (const double*)pc, pn, x, c->S, track, it, (int)(it + 1 == max_iter)),
+                            "cg: kernel launch");
+            else
+                HS_TRY_CUDA(launch_dependent(k_cg_pupdate, c->grid, kCgBlock, c->stream, nn, (const double*)c->r, c->p,
+                                             c->S, track),
+                            "cg: kernel launch");
             HS_CHECK_LAUNCH("cg: direction kernel");
         }
         enqueued += todo;

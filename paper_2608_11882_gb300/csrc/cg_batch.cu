@@ -164,6 +164,10 @@ __global__ void __launch_bounds__(NT, MINB) k_cgb_spmv_dot(const SysDev* sys, in
     }
 }
 
+// WITH_X: x += alpha p too, as k_cg_update; batches with a large system leave that to
+// k_cgb_direction (80 bytes per row and iteration instead of 88: one of 200^3
+// 123.7 -> 107.5 ms, 16 CSR systems of 64^3 116 -> 128).
+template <bool WITH_X>
 __global__ void __launch_bounds__(kCgBlock) k_cgb_update(const SysDev* sys, int nsys)
 {
     grid_dependency_wait();
@@ -172,8 +176,9 @@ __global__ void __launch_bounds__(kCgBlock) k_cgb_update(const SysDev* sys, int 
     if (*(volatile int32_t*)&s.S->done || s.S->iters >= s.max_iter) return;
     __shared__ double sh[kCgBlock / 32];
     const double alpha = s.S->alpha;
-    const double rr = cg_update_rows(s.A.n, s.r, s.q, alpha, (int64_t)local * kCgBlock + threadIdx.x,
-                                     (int64_t)s.nblocks * kCgBlock);
+    const int64_t t0 = (int64_t)local * kCgBlock + threadIdx.x, stride = (int64_t)s.nblocks * kCgBlock;
+    const double rr = WITH_X ? cg_update_xr_rows(s.A.n, s.x, s.r, s.p, s.q, alpha, t0, stride)
+                             : cg_update_rows(s.A.n, s.r, s.q, alpha, t0, stride);
     allow_dependents();
     const double blk = block_sum<kCgBlock>(rr, sh);
     if (!arrive_last_sys(blk, s.partials, &s.S->ticket, local, s.nblocks)) return;
@@ -205,6 +210,21 @@ __global__ void __launch_bounds__(kCgBlock) k_cgb_direction(const SysDev* sys, i
                                                  (int64_t)local * kCgBlock + threadIdx.x, (int64_t)s.nblocks * kCgBlock);
     allow_dependents();
     if (s.mode == SP_STAGED && next) cg_fold_pmax(pm, s.S, (it + 1) % 3, local == 0);
+}
+
+// p = r + beta p.
+__global__ void __launch_bounds__(kCgBlock) k_cgb_pupdate(const SysDev* sys, int nsys)
+{
+    grid_dependency_wait();
+    int local;
+    const SysDev& s = sys[sys_of_block(sys, nsys, &local)];
+    // the update kernel of this iteration has already counted it
+    if (*(volatile int32_t*)&s.S->done) return;
+    const double beta = s.S->beta;
+    const unsigned pm = cg_pupdate_rows(s.A.n, s.r, s.p, beta, (int64_t)local * kCgBlock + threadIdx.x,
+                                        (int64_t)s.nblocks * kCgBlock);
+    allow_dependents();
+    if (s.mode == SP_STAGED) cg_fold_pmax(pm, s.S, s.S->iters % 3, local == 0);
 }
 
 // ||b - A x||^2 into rr_true (q = A x from k_cgb_apply_x).
@@ -246,6 +266,7 @@ struct hs_cg_batch {
     std::vector<int32_t> big;  // their places in the batch
     int32_t total_blocks;
     bool has_mode[3];          // SpmvModes present (one SpMV kernel each)
+    bool x_late;               // x is updated with p, not with r: some system is large (cg_x_late)
     std::vector<SysDev> sys;   // host copy (b, x filled per run)
     SysDev* d_sys;
     // small matrix-free systems, solved whole in one launch (cg_small.cu)
@@ -303,6 +324,7 @@ static int cg_batch_fill(hs_cg_batch* b, const hs_op* ops, int32_t n)
         s.mode = spmv_mode(s.A, s.nblocks);
         s.nshares = s.mode == SP_STAGED ? spmv_shares(s.nblocks) : s.nblocks;
         b->has_mode[s.mode] = true;
+        if (cg_x_late(s.A)) b->x_late = true;
         s.block0 = (int32_t)blocks;
         blocks += s.nblocks;
         part_total += 2 * (int64_t)s.nblocks;
@@ -489,10 +511,15 @@ int cg_batch_run(hs_cg_batch_t b, const void* const* bs, void* const* xs, double
             }
             if (b->has_mode[SP_ROWS]) CGB_LAUNCH_DEP((k_cgb_spmv_dot<SP_ROWS, kCgBlock, 1>), "cg batch: spmv+dot kernel");
             if (b->has_mode[SP_CSR]) CGB_LAUNCH_DEP((k_cgb_spmv_dot<SP_CSR, kCgBlock, 1>), "cg batch: spmv+dot kernel");
-            CGB_LAUNCH_DEP(k_cgb_update, "cg batch: update kernel");
-            HS_TRY_CUDA(launch_dependent(k_cgb_direction, G, kCgBlock, b->stream, b->d_sys, nbig, enqueued + t),
-                        "cg batch: kernel launch");
-            HS_CHECK_LAUNCH("cg batch: direction kernel");
+            if (b->x_late) {
+                CGB_LAUNCH_DEP(k_cgb_update<false>, "cg batch: update kernel");
+                HS_TRY_CUDA(launch_dependent(k_cgb_direction, G, kCgBlock, b->stream, b->d_sys, nbig, enqueued + t),
+                            "cg batch: kernel launch");
+                HS_CHECK_LAUNCH("cg batch: direction kernel");
+            } else {
+                CGB_LAUNCH_DEP(k_cgb_update<true>, "cg batch: update kernel");
+                CGB_LAUNCH_DEP(k_cgb_pupdate, "cg batch: p update kernel");
+            }
         }
         enqueued += todo;
         if (chunk < 32) chunk *= 2;

@@ -450,6 +450,63 @@ __device__ __forceinline__ double cg_update_rows(int64_t n, double* __restrict__
     return rr;
 }
 
+// x += alpha p, r -= alpha q; returns this thread's share of r.r.
+__device__ __forceinline__ double cg_update_xr_rows(int64_t n, double* __restrict__ x, double* __restrict__ r,
+                                                    const double* __restrict__ p, const double* __restrict__ q,
+                                                    double alpha, int64_t t0, int64_t stride)
+{
+    double rr = 0.0;
+    const int64_t npairs = n >> 1;
+    const bool xvec = (reinterpret_cast<uintptr_t>(x) & 15) == 0;
+    for (int64_t t = t0; t < npairs; t += stride) {
+        const double2 pv = reinterpret_cast<const double2*>(p)[t];
+        const double2 qv = reinterpret_cast<const double2*>(q)[t];
+        double2 xv = xvec ? reinterpret_cast<double2*>(x)[t] : make_double2(x[2 * t], x[2 * t + 1]);
+        double2 rv = reinterpret_cast<double2*>(r)[t];
+        xv.x = __fma_rn(alpha, pv.x, xv.x);
+        xv.y = __fma_rn(alpha, pv.y, xv.y);
+        rv.x = __fma_rn(-alpha, qv.x, rv.x);
+        rv.y = __fma_rn(-alpha, qv.y, rv.y);
+        if (xvec) {
+            reinterpret_cast<double2*>(x)[t] = xv;
+        } else {
+            x[2 * t] = xv.x;
+            x[2 * t + 1] = xv.y;
+        }
+        reinterpret_cast<double2*>(r)[t] = rv;
+        rr = __fma_rn(rv.x, rv.x, rr);
+        rr = __fma_rn(rv.y, rv.y, rr);
+    }
+    if ((n & 1) && t0 == 0) {
+        x[n - 1] = __fma_rn(alpha, p[n - 1], x[n - 1]);
+        const double rt = __fma_rn(-alpha, q[n - 1], r[n - 1]);
+        r[n - 1] = rt;
+        rr = __fma_rn(rt, rt, rr);
+    }
+    return rr;
+}
+
+// p = r + beta p; returns the largest |p| high word of this thread's values.
+__device__ __forceinline__ unsigned cg_pupdate_rows(int64_t n, const double* __restrict__ r, double* __restrict__ p,
+                                                    double beta, int64_t t0, int64_t stride)
+{
+    unsigned pm = 0;
+    const int64_t npairs = n >> 1;
+    for (int64_t t = t0; t < npairs; t += stride) {
+        const double2 a = reinterpret_cast<const double2*>(p)[t];
+        const double2 b = reinterpret_cast<const double2*>(r)[t];
+        const double2 v = make_double2(__fma_rn(beta, a.x, b.x), __fma_rn(beta, a.y, b.y));
+        reinterpret_cast<double2*>(p)[t] = v;
+        pm = max(pm, max(xs_abs_hi(v.x), xs_abs_hi(v.y)));
+    }
+    if ((n & 1) && t0 == 0) {
+        const double v = __fma_rn(beta, p[n - 1], r[n - 1]);
+        p[n - 1] = v;
+        pm = max(pm, xs_abs_hi(v));
+    }
+    return pm;
+}
+
 // What a direction pass does to x, which waits for nothing and so is updated
 // where its direction is read anyway: nothing, x += alpha p, or the steps of
 // two iterations at once, x += alpha0 p0 and then x += alpha p (p0 the direction
@@ -521,6 +578,22 @@ __device__ __forceinline__ void cg_fold_pmax(unsigned m, CgScalars* S, int slot,
     }
 }
 
+// The same with one atomic per block, for passes of few blocks, where every warp
+// comes before the slot holds anything: 8 x 100 x 100 2263 -> 2160 us per solve.
+__device__ __forceinline__ void cg_fold_pmax_block(unsigned m, CgScalars* S, int slot, bool first_block)
+{
+    __shared__ unsigned wmax[kCgBlock / 32];
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        unsigned b = 0;
+        for (int w = 0; w < kCgBlock / 32; ++w) b = max(b, wmax[w]);
+        atomicMax(&S->pmax[slot], (unsigned long long)b << 32);
+        if (first_block) S->pmax[(slot + 1) % 3] = 0;
+    }
+}
+
 struct CgMixed;   // mixed-precision state (cg_mixed.cu)
 
 // The TMA-staged form of the SP_STAGED SpMV (cg_spmv_tma.cu) for single
@@ -537,10 +610,11 @@ int check_op(const hs_op* A);
 OpDev to_dev(const hs_op* A);
 int grid_for(int64_t n);
 size_t cg_partials(const OpDev& A, int grid);
-// Whether a solve keeps two direction buffers and updates x every second
-// iteration (76 bytes per row and iteration instead of 80): vectors beyond L2,
-// where bytes count.
-inline bool cg_two_directions(const OpDev& A) { return A.n >= ((int64_t)1 << 22); }
+// Whether a solve adds to x in the direction pass instead of the update pass, and
+// for two iterations at a time (76 bytes per row and iteration, where the update
+// pass's form moves 88): vectors beyond L2, where bytes count.  Solves that stay in
+// L2 are bound by latency (k_cg_update).  162^3, 4.25 M: 49.4 -> 47.2 ms.
+inline bool cg_x_late(const OpDev& A) { return A.n >= ((int64_t)1 << 22); }
 int cg_create_vectors(hs_cg_t* out, const hs_op* A, void* stream, bool need_p);
 int launch_apply(const OpDev& A, const double* p, double* y, cudaStream_t s);
 
@@ -553,7 +627,7 @@ struct hs_cg {
     double* r;
     double* p;
     double* q;
-    double* p2;            // second direction buffer (cg_two_directions), else NULL
+    double* p2;            // second direction buffer (cg_x_late), else NULL
     void* arena;           // device allocation behind ctl, S, partials, r, p and q; null: the caller's scratch
     char* ctl;             // control words of the small-system kernel (cg_small.cuh), S among them
     double* partials;      // cg_partials(A, grid) doubles

@@ -231,7 +231,6 @@ __global__ void __launch_bounds__(kSpBlock, 5)
             S->done = 2;   // breakdown: A is not positive definite on p
         } else {
             S->alpha = S->rho / tot;
-            S->alpha2[S->iters & 1] = S->alpha;
         }
     }
 }
