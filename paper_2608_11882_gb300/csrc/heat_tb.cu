@@ -74,6 +74,9 @@ struct TbShape {
     static constexpr int RW = W * V;
     static constexpr int TX = RW - 2 * H;
     static constexpr int RT = 2;
+    // Shared planes a level keeps: two in turn, or in FP32 as many as the ring has
+    // stages, in the ring's slots (constants there; FIXED64 at depth 4 loses 3%)
+    static constexpr int LEV = std::is_same<T, float>::value ? 3 : 2;
     // FP32 warp rows: 16 (64 registers, two blocks of 16 warps per SM at depth 2);
     // the halo rows weigh less than with 12: 512^3 125.0 -> 123.1 us per step,
     // 1000^3 828 -> 767, at depth 4 143 -> 128.  Wider types, and rows of 34
@@ -158,6 +161,9 @@ __device__ __forceinline__ unsigned long long tb_chunk(const CUtensorMap* map, T
     // lanes that start and end a warp would have to load theirs (157 us at 512^3
     // against 133, with spills).
     constexpr bool F32 = std::is_same<T, float>::value;
+    // FIXED64 at depth 4 counts its slots: 512^3 13.69 ms per 24 steps, against 14.41
+    // in turns (96^3 0.50 and 0.55); depths 2 and 3 gain 2 to 3% by the turns
+    constexpr bool TURNS = !(kIsFixed<T> && L == 4);
     static_assert(L <= H, "end columns are not part of the tile");
     const int tx = threadIdx.x, ty = threadIdx.y;
     const int tid = ty * W + tx;
@@ -196,11 +202,11 @@ __device__ __forceinline__ unsigned long long tb_chunk(const CUtensorMap* map, T
 
     // plane q in slot s_cur of the ring; false: the march ends
     auto step = [&](int q, int s_cur, uint32_t phase) -> bool {
-        if (!mbar_wait_quick(&bars[s_cur], phase)) {
+        if (!(TURNS ? mbar_wait_quick(&bars[s_cur], phase) : mbar_wait_bounded(&bars[s_cur], phase))) {
             atomicExch(err, 1);
             *s_abort = 1;
         }
-        const int s_prev = (s_cur + NST - 1) % NST;   // plane q-1 (junk at q = q0)
+        const int s_prev = s_cur == 0 ? NST - 1 : s_cur - 1;   // plane q-1 (junk at q = q0)
         T up[RT][V];
 #pragma unroll
         for (int j = 0; j < RT; ++j) ld_vec(stage + s_cur * PLANE + own + j * BW, up[j]);
@@ -208,7 +214,7 @@ __device__ __forceinline__ unsigned long long tb_chunk(const CUtensorMap* map, T
         for (int t = 1; t <= L; ++t) {
             const int p = q - t;
             const T* src = (t == 1) ? stage + s_prev * PLANE + own
-                                    : lev + ((t - 2) * NST + s_prev) * PLANE + own;
+                                    : lev + ((t - 2) * S::LEV + (F32 ? s_prev : (q - 1) & 1)) * PLANE + own;
             T ym[V], yp[V], v[RT][V];
             ld_vec(src - BW, ym);
             ld_vec(src + RT * BW, yp);
@@ -230,12 +236,16 @@ __device__ __forceinline__ unsigned long long tb_chunk(const CUtensorMap* map, T
                     f32_row_update(c, left, right, yl, yh, zb[t - 1][j], up[j], r, v[j]);
                 } else {
 #pragma unroll
-                    for (int i = 0; i < V; ++i)
-                        v[j][i] = Point<T, EXACT>::update(c[i], i == 0 ? left : c[i - 1],
-                                                          i == V - 1 ? right : c[i + 1], yl[i], yh[i],
-                                                          zb[t - 1][j][i], up[j][i], r, t == 1 ? ks : 0);
+                    for (int i = 0; i < V; ++i) {
+                        const T w = Point<T, EXACT>::update(c[i], i == 0 ? left : c[i - 1],
+                                                            i == V - 1 ? right : c[i + 1], yl[i], yh[i],
+                                                            zb[t - 1][j][i], up[j][i], r, t == 1 ? ks : 0);
+                        // masked where it is formed: FIXED64 at depth 3 runs 2 to 4% faster than with
+                        // the FP32 rows' separate loop below
+                        v[j][i] = !MASK || (zin && in_x[i] && in_y[j]) ? w : T(0);
+                    }
                 }
-                if constexpr (MASK) {   // Dirichlet zeros outside the interior
+                if constexpr (MASK && F32 && !EXACT) {   // Dirichlet zeros outside the interior
 #pragma unroll
                     for (int i = 0; i < V; ++i)
                         if (!(zin && in_x[i] && in_y[j])) v[j][i] = T(0);
@@ -249,7 +259,7 @@ __device__ __forceinline__ unsigned long long tb_chunk(const CUtensorMap* map, T
                     zc[t - 1][j][i] = up[j][i];
                 }
             if (t < L) {
-                T* lp = lev + ((t - 1) * NST + s_cur) * PLANE + own;
+                T* lp = lev + ((t - 1) * S::LEV + (F32 ? s_cur : q & 1)) * PLANE + own;
 #pragma unroll
                 for (int j = 0; j < RT; ++j) {
                     st_vec(lp + j * BW, v[j]);
@@ -297,10 +307,22 @@ __device__ __forceinline__ unsigned long long tb_chunk(const CUtensorMap* map, T
     // 129.2 -> 125.0 us per step against a loop that counts its slots)
     static_assert(NST == 3, "a turn visits each slot once");
     uint32_t phase = 0;
-    for (int q = q0;; q += 3, phase ^= 1u) {
-        if (!step(q, 0, phase)) break;
-        if (!step(q + 1, 1, phase)) break;
-        if (!step(q + 2, 2, phase)) break;
+    if constexpr (TURNS) {
+        for (int q = q0;; q += 3, phase ^= 1u) {
+            if (!step(q, 0, phase)) break;
+            if (!step(q + 1, 1, phase)) break;
+            if (!step(q + 2, 2, phase)) break;
+        }
+    } else {
+        int s_cur = 0;
+#pragma unroll 3
+        for (int q = q0; q <= qlast; ++q) {
+            if (!step(q, s_cur, phase)) break;
+            if (++s_cur == NST) {
+                s_cur = 0;
+                phase ^= 1u;
+            }
+        }
     }
     return mx;
 }
@@ -314,8 +336,8 @@ __global__ void __launch_bounds__(TbShape<T, L, W>::NT, MINB)
     static_assert(S::TY > 0 && S::TX > 0, "tile too small for the temporal depth");
     extern __shared__ __align__(128) unsigned char smem_raw[];
     T* stage = reinterpret_cast<T*>(smem_raw);
-    T* lev = stage + NST * S::PLANE;   // level t (1..L-1), slot s: lev + ((t-1) * NST + s) * PLANE
-    uint64_t* bars = reinterpret_cast<uint64_t*>(lev + (L - 1) * NST * S::PLANE);
+    T* lev = stage + NST * S::PLANE;   // level t (1..L-1), slot s: lev + ((t-1) * LEV + s) * PLANE
+    uint64_t* bars = reinterpret_cast<uint64_t*>(lev + (L - 1) * S::LEV * S::PLANE);
     __shared__ int s_abort;
 
     const int tid = threadIdx.y * W + threadIdx.x;
@@ -371,7 +393,7 @@ int tb_launch_w(const TbCall& c)
     constexpr int MINB = L == 2 ? 2 : 1;
     using S = TbShape<T, L, W>;
     constexpr size_t smem =
-        sizeof(T) * (size_t)NST * L * S::PLANE + NST * sizeof(uint64_t);
+        sizeof(T) * (size_t)(NST + S::LEV * (L - 1)) * S::PLANE + NST * sizeof(uint64_t);
     if (c.box[0] != (uint32_t)S::BW || c.box[1] != (uint32_t)S::ROWS)
         return fail(HS_EINVAL, "heat: tensor map box %ux%u does not match the kernel's %dx%d", c.box[0],
                     c.box[1], S::BW, S::ROWS);
