@@ -646,9 +646,14 @@ int pick_kc_tb(const HeatGeom& g, int arith, int L)
         const int64_t blocks = tiles * ((g.nz + kc - 1) / kc);
         return (blocks + slots - 1) / slots * (kc + 2 * L + 3);
     };
-    // a launch holds 65535 chunks
+    // A grid too small to fill the GPU with chunks of 8 L planes takes chunks of 4 L
+    // and up: with one wave or less, the planes of one chunk are the time of a pass
+    // (96^3, 24 steps: FP32 at depth 2 240 -> 152 us, where tiles of 28 rows had made
+    // it slower than those of 20 at 225; FIXED64 at depth 4 497 -> 311).
+    // A launch holds 65535 chunks.
     const int64_t fit = ((int64_t)g.nz + 65534) / 65535;
-    const int64_t shortest = std::max(fit, std::min<int64_t>(g.nz, 8 * L)), longest = std::min<int64_t>(g.nz, 64 * L);
+    const int64_t floor_kc = tiles * ((g.nz + 8 * L - 1) / (8 * L)) < slots ? 4 * L : 8 * L;
+    const int64_t shortest = std::max(fit, std::min<int64_t>(g.nz, floor_kc)), longest = std::min<int64_t>(g.nz, 64 * L);
     const int64_t chunks = (12 * (int64_t)kNumSMs + tiles - 1) / tiles;
     int64_t best = std::max(shortest, (g.nz + chunks - 1) / chunks);
     int64_t least = planes(best) * 19 / 20;
