@@ -694,20 +694,42 @@ int pick_kc_stream(const HeatGeom& g, int arith)
     return (int)kc;
 }
 
-// Whether heat_step advances this handle with the multi-step kernel: grids
-// below 2^22 points, 2^23 in FP32, unless the caller asked for another schedule
-// or depth.  Measured per step, Interior + Boundary launches (FP32: the blocked
-// pass) against it: 64^3 FP64 14.4 / 3.5 us, FP32 9.3 / 2.5; 128^3 FP64 18.5 /
-// 12.2, FP32 10.3 / 6.0; 160^3 FP64 27.5 / 23.6, FIXED64 24.7 / 19.6, FP32 13.4
-// / 8.0; 176^3 FP64 29.5 / 31.1, FIXED64 24.7 / 25.5; 192^3 FP32 13.4 / 10.7;
-// 208^3 FP32 13.4 / 15.4.
+// Whether heat_step advances this handle with the multi-step kernel, unless the
+// caller asked for another schedule or depth.  Its time goes with its bricks, the
+// streaming kernel's and the blocked pass's only above a floor; thin grids leave
+// bricks and tiles alike partly empty.  Per step, launches / multi-step kernel:
+//   FP64, to 24 bricks per SM: 64^3 14.4 / 3.4 us, 160^3 28.3 / 22.5, 500 x 9 x 900
+//     (3600) 33.8 / 32.3; 66 x 200 x 310 (3900) 35.7 / 36.0, 20 x 400 x 400 (5000)
+//     43.8 / 45.6, 16 x 640 x 400 (8000) 63.6 / 74.7.  From 2^22 points 176^3 (2904)
+//     28.0 / 30.7.
+//   FIXED64, to 40: 160^3 24.7 / 19.5, 20 x 400 x 400 43.7 / 39.0; 17 x 600 x 380
+//     (7125) 57.3 / 58.7.  From 2^22 points 176^3 25.3 / 25.8.
+//   FP32 against the blocked pass, four steps deep, to 6: 64^3 7.3 / 2.6, 128^3 7.2 /
+//     6.1, 60 x 200 x 260 (845) 7.8 / 6.4; 144^3 (972) 7.3 / 7.8, 160^3 7.3 / 8.2, 65
+//     x 340 x 340 (3740) 13.4 / 23.0.  Two deep (tb_deep), to 9: 250 x 140 x 140
+//     (1260) 10.3 / 8.8; 370 x 120 x 120 (1440) 10.3 / 11.2.  Thin grids, whose tiles
+//     hold 7/4 of the bricks' points and more: 60 x 260 x 260 (1105) 8.8 / 8.2, 16 x
+//     640 x 400 (4000) 24.7 / 17.4; from 2^22 points only the narrowest: 20 x 600 x 600
+//     30.3 / 27.6, 60 x 360 x 370 13.4 / 18.8; 640 x 640 x 10, mostly z halo, 10.4 / 7.6.
+//   FP32 one step at a time (tdepth 1): 192^3 15.9 / 10.7, 65 x 340 x 340 22.8 / 22.5.
 bool use_multi(const hs_heat_desc* d, const hs_heat* h)
 {
     if (d->flags & (HS_SCHED_FULL | HS_VARKAPPA)) return false;
     if (h->arith != A_F32 && h->arith != A_FX64 && h->arith != A_F64_XS) return false;
     if (d->tdepth > 1) return false;   // the caller asked for temporal blocking
-    const int64_t npts = (int64_t)h->g.nx * h->g.ny * h->g.nz;
-    return npts < ((int64_t)1 << (h->arith == A_F32 ? 23 : 22));
+    const HeatGeom& g = h->g;
+    const int64_t npts = (int64_t)g.nx * g.ny * g.nz, bricks = multi_bricks(h->arith, g);
+    const bool below22 = npts < ((int64_t)1 << 22);
+    if (h->arith == A_F64_XS) return below22 && bricks <= 24 * kNumSMs;
+    if (h->arith == A_FX64) return below22 && bricks <= 40 * kNumSMs;
+    if (npts >= ((int64_t)1 << 23)) return false;
+    if (d->tdepth == 1 || bricks <= (h->deep ? 6 : 9) * kNumSMs || g.nx <= 24) return true;
+    int TX = 0, TY = 0;
+    const int L = h->deep ? 4 : 2;
+    tb_tile(A_F32, L, g.nx, &TX, &TY);
+    const int64_t tiles =
+        (int64_t)((g.nx + TX - 1) / TX) * TX * ((g.ny + TY - 1) / TY) * TY * ((int64_t)g.nz + 2 * L + 3);
+    return below22 && 7 * 4096 * bricks <= 4 * tiles;
 }
 
 // n_steps steps in one launch of the multi-step kernel.

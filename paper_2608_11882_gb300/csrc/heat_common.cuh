@@ -348,6 +348,9 @@ struct MultiCall {
     cudaStream_t stream;
 };
 int multi_launch(const MultiCall& c);
+// Bricks a grid takes in the multi-step kernel: of 2048 points, 4096 in FP32.
+int64_t multi_bricks(int arith, const HeatGeom& g);
+
 // What the batched kernel needs to know about a heat handle (heat.cu).
 struct HeatBatchView {
     HeatGeom g;

@@ -296,7 +296,7 @@ int multi_launch_t(const MultiCall& c)
     a.steps = c.steps;
     a.tiles_x = (g.nx + kMuTW - 1) / kMuTW;
     a.tiles_y = (g.ny + S::ROWS - 1) / S::ROWS;
-    a.bricks = a.tiles_x * a.tiles_y * ((g.nz + kMuKZ - 1) / kMuKZ);
+    a.bricks = (int)multi_bricks(c.arith, g);
     a.bar = (unsigned long long*)c.sync;
     a.err = c.err;
     const int blocks = std::min(a.bricks, slots);
@@ -309,6 +309,12 @@ int multi_launch_t(const MultiCall& c)
     }
     HS_CHECK_LAUNCH("heat multi-step kernel");
     return HS_OK;
+}
+
+int64_t multi_bricks(int arith, const HeatGeom& g)
+{
+    const int rows = arith == A_F32 ? MultiShape<float>::ROWS : MultiShape<double>::ROWS;
+    return (int64_t)((g.nx + kMuTW - 1) / kMuTW) * ((g.ny + rows - 1) / rows) * ((g.nz + kMuKZ - 1) / kMuKZ);
 }
 
 int multi_launch(const MultiCall& c)
