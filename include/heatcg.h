@@ -188,8 +188,8 @@ int heat_upload(hs_heat_t h, const void* u, int src_is_device);
  * and passes of four steps are faster, it takes those while four steps remain.  Small grids of the default arithmetics (to 2^22
  * points, 2^23 for HS_F32, where it is faster; HS_F64, HS_F32 or HS_FIXED64 with
  * tdepth 0 or 1, without HS_SCHED_FULL or HS_VARKAPPA, heat_time_interior off) run
- * all n_steps in one cooperative launch whose blocks meet at a barrier after every
- * step, with the same result bit for bit.  The result equals stepping one step at a time up to
+ * up to 1024 steps in one cooperative launch whose blocks meet at a barrier after
+ * every step, with the same result bit for bit.  The result equals stepping one step at a time up to
  * rounding (bit for bit for FP32, and for FP64 against an HS_FP64_PIPE handle
  * stepped one step at a time, whose per-point arithmetic is the same; FIXED64
  * may rescale at different steps).  Asynchronous: launch errors

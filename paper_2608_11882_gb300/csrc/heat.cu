@@ -694,6 +694,11 @@ int pick_kc_stream(const HeatGeom& g, int arith)
     return (int)kc;
 }
 
+// Steps of one launch of the multi-step kernel, whose blocks may fill the GPU: at
+// 3 to 40 us per step other streams' kernels wait 40 ms at most, and a launch in
+// 1024 steps costs less than 0.2%.
+constexpr int64_t kMultiSteps = 1024;
+
 // Whether heat_step advances this handle with the multi-step kernel, unless the
 // caller asked for another schedule or depth.  Its time goes with its bricks, the
 // streaming kernel's and the blocked pass's only above a floor; thin grids leave
@@ -1147,7 +1152,7 @@ int heat_step(hs_heat_t h, int64_t n_steps)
     if (n_steps < 0) return fail(HS_EINVAL, "heat_step: n_steps = %lld < 0", (long long)n_steps);
     if (h->msync && !h->timing) {
         while (n_steps > 0) {
-            const int part = (int)std::min<int64_t>(n_steps, (int64_t)1 << 20);
+            const int part = (int)std::min<int64_t>(n_steps, kMultiSteps);
             const int rc = multi_steps(h, part);
             if (rc != HS_OK) return rc;
             n_steps -= part;

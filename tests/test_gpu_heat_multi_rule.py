@@ -38,3 +38,19 @@ def test_line_and_results(arith, shape, one):
                 assert (launches == 1) == one
             out.append(h.read(torch.empty_like(u0)))
     assert torch.equal(out[0], out[1])
+
+
+def test_long_runs_are_cut_into_launches():
+    """A launch holds the GPU for 1024 steps at most; the parts go on from one another."""
+    pkg, torch = lib(), require_cuda()
+    from paper_2608_11882_gb300 import _native as native
+    u0 = torch.from_numpy(np.random.default_rng(2).uniform(-1, 1, size=(9, 11, 70))).cuda()
+    out = []
+    for extra in (0, pkg.HS_SCHED_FULL):
+        with pkg.Heat(70, 11, 9, 0.02, flags=extra) as h:
+            h.upload(u0)
+            before = native.launch_count()
+            h.step(2500)
+            assert native.launch_count() - before == (2500 if extra else 3)
+            out.append(h.read(torch.empty_like(u0)))
+    assert torch.equal(out[0], out[1])
