@@ -374,7 +374,8 @@ int cg_spmv(const hs_op* A, const void* p, void* q, int kernel, double* pq, void
 /* Create a CG context: checks A, takes a device copy of A's arrays when
  * A->host == 1 (otherwise it keeps A's device pointers, which must outlive
  * the context), and allocates the workspace (r, p, q, reduction partials and
- * device scalars).  Errors: HS_EINVAL, HS_ENOMEM, HS_ECUDA. */
+ * device scalars; from 2^22 unknowns a second buffer for p where the memory
+ * allows, which saves reading and writing x in every second iteration).  Errors: HS_EINVAL, HS_ENOMEM, HS_ECUDA. */
 int cg_create(hs_cg_t* out, const hs_op* A, void* stream);
 
 /* Solve A x = b by unpreconditioned FP64 CG (textbook form, Section 7.5):

@@ -464,8 +464,14 @@ int cg_create_vectors(hs_cg_t* out, const hs_op* A, void* stream, bool need_p)
     auto align = [](size_t x) { return (x + 255) & ~(size_t)255; };
     const size_t s_ctl = align(sizeof(CgSmallCtl)), s_part = align(sizeof(double) * cg_partials(c->A, c->grid));
     const size_t s_vec = align(sizeof(double) * (size_t)cg_vector_len(c->A));
-    const bool two = need_p && cg_x_late(c->A);
-    CG_ALLOC(c->arena, s_ctl + s_part + (two ? 4 : need_p ? 3 : 2) * s_vec);
+    // large solves keep two directions where the memory allows
+    bool two = need_p && cg_x_late(c->A);
+    if (two && dev_alloc(&c->arena, s_ctl + s_part + 4 * s_vec, c->stream) != cudaSuccess) {
+        (void)cudaGetLastError();
+        c->arena = nullptr;
+        two = false;
+    }
+    if (!two) CG_ALLOC(c->arena, s_ctl + s_part + (need_p ? 3 : 2) * s_vec);
     c->ctl = (char*)c->arena;
     c->S = &((CgSmallCtl*)c->ctl)->S;
     c->partials = (double*)(c->ctl + s_ctl);

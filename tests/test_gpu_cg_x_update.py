@@ -2,6 +2,10 @@
 update pass for systems that stay in L2, in the direction pass for large ones
 and for every system of a batch that holds a large one.  The values are the
 same, so results agree bit for bit wherever the solve stops."""
+import os
+import subprocess
+import sys
+
 import numpy as np
 import pytest
 
@@ -58,3 +62,41 @@ def test_large_csr_keeps_two_directions(max_iter):
     assert i1["iters"] == i2[0]["iters"] and i1["converged"] == (max_iter == 2000)
     assert torch.equal(x1, x2[0])
     assert abs(i1["relres_recur"] - i1["relres_true"]) <= 1e-9 * max(1.0, i1["relres_true"])
+
+
+# a process of its own: its memory pool holds nothing from other solves
+ONE_BUFFER = """
+import torch, paper_2608_11882_gb300 as pkg
+n = 400
+op = pkg.Operator.stencil(n, n, n)
+b = torch.randn(n ** 3, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(3))
+out = []
+for its in (1, 6, 7):
+    x = torch.zeros_like(b)
+    with pkg.CG(op) as cg:
+        out.append((x, cg.run(b, x, rtol=1e-3, max_iter=its)[1]))
+vec = 8 * n ** 3
+second = [torch.zeros_like(b) for _ in out]
+torch.cuda.synchronize()
+torch.cuda.empty_cache()
+fill = torch.empty(torch.cuda.mem_get_info()[0] - 7 * vec // 2, dtype=torch.uint8, device="cuda")
+assert 3 * vec < torch.cuda.mem_get_info()[0] < 4 * vec
+for its, x, (x0, i0) in zip((1, 6, 7), second, out):
+    with pkg.CG(op) as cg:
+        _, info = cg.run(b, x, rtol=1e-3, max_iter=its)
+    assert torch.equal(x, x0) and info == i0 and info["iters"] == its, (info, i0)
+print("same")
+"""
+
+
+def test_one_direction_buffer_where_memory_is_short():
+    """Room for r, q and one direction: the solve keeps one buffer and gives the
+    same result bit for bit."""
+    torch = require_cuda()
+    lib()
+    if torch.cuda.mem_get_info()[0] < 24 << 30:
+        pytest.skip("needs 24 GB of device memory")
+    torch.cuda.empty_cache()
+    root = os.path.dirname(os.path.dirname(os.path.abspath(__file__)))
+    r = subprocess.run([sys.executable, "-c", ONE_BUFFER], cwd=root, capture_output=True, text=True, timeout=300)
+    assert r.returncode == 0 and r.stdout.split() == ["same"], r.stderr[-2000:]
