@@ -156,7 +156,9 @@ int heat_buffer_bytes(const hs_heat_desc* desc, size_t* bytes);
 
 /* Device bytes heat_create would allocate for desc (for admission control):
  * the two field buffers unless the caller supplies them, and the per-step
- * state of the exact-sum and FIXED64 arithmetics (and kappa and dt f for HS_VARKAPPA, two fields' worth). */
+ * state of the exact-sum and FIXED64 arithmetics (and kappa and dt f for
+ * HS_VARKAPPA, two fields' worth).  Not counted: the rest of a handle's words and
+ * the rounding of the buffers to 256 bytes, less than 1.5 KiB together. */
 int heat_device_bytes(const hs_heat_desc* desc, size_t* bytes);
 
 /* Load the interior field u (nx*ny*nz elements of the handle's dtype, x

@@ -14,12 +14,6 @@ constexpr int kCgSmallMaxBricks = 4096;  // bricks of one system
 // (the kernel would take about 12 us per iteration there too, against 16).
 constexpr int64_t kCgSmallMinN = (int64_t)1 << 14, kCgSmallMaxN = (int64_t)1 << 22;
 constexpr int kCgSmallMinNx = 16;        // also bounds what the padding of odd rows adds
-// Values each of r, p and q holds for a system of n unknowns.
-inline int64_t cg_vector_len(const OpDev& A)
-{
-    return A.kind == HS_OP_STENCIL7 ? (int64_t)((A.nx + 1) & ~1) * A.ny * A.nz : (A.n + 1) & ~(int64_t)1;
-}
-
 struct CgSmallSys {
     int32_t nx, ny, nz;
     int32_t lg;                  // log2 of the threads per brick row: 5 (64 x 8 x 4) or 4 (32 x 16 x 4)
@@ -54,6 +48,12 @@ struct CgSmallCtl {
 
 // Fills the geometry of a system that takes this path; false for any other.
 bool cg_small_shape(const OpDev& A, CgSmallSys* s);
+// Values each of r, p and q holds: rows of even pitch on this path, else n, made even.
+inline int64_t cg_vector_len(const OpDev& A)
+{
+    CgSmallSys s;
+    return cg_small_shape(A, &s) ? (int64_t)s.pitch * A.ny * A.nz : (A.n + 1) & ~(int64_t)1;
+}
 // One launch over ngroups groups, one after the other.  single: one system in
 // all; bricks: of the largest group.  *err is set to 1 when a bounded wait ran out.
 int cg_small_launch(const CgSmallSys* sys, const CgSmallGroup* groups, int ngroups, bool single, int64_t bricks,

@@ -70,15 +70,19 @@ class Result:
 
 
 def device_bytes(req: Request) -> int:
-    """Device memory a request holds while admitted (both padded field buffers
-    and, for FP64, the 64-byte per-step state, for heat; r, p, q, b and x for
-    CG), with row padding to 128 bytes."""
+    """Device memory a request holds while admitted: for heat both padded field
+    buffers (rows of 128 bytes) and the handle's words; for CG b, x, r, q, p (rows
+    of even length where the one-launch solve pads them), from 2^22 unknowns the
+    second p, and at most 68 KiB of reduction partials and control words."""
     nz, ny, nx = req.shape
     if req.kind == "heat":
         elem = 8 if req.dtype == "f64" else 4
         pitch = -(-(32 // elem + nx + 1) * elem // 128) * 128
-        return 2 * pitch * (ny + 2) * (nz + 2) + (64 if req.dtype == "f64" else 0)
-    return 5 * 8 * req.points
+        return 2 * (-(-pitch * (ny + 2) * (nz + 2) // 256) * 256) + 1024
+    n = req.points
+    padded = nx % 2 and nx >= 16 and 1 << 14 <= n < 1 << 22
+    vectors = 4 if n >= 1 << 22 else 3
+    return 8 * (2 * n + vectors * (n + ny * nz if padded else n + 32)) + (68 << 10)
 
 
 def kbar(samples) -> float:
