@@ -868,7 +868,7 @@ def serving_side(args, loads=(0.5, 0.7, 0.9)):
     base = poisson_trace(args.requests, rate=1.0, seed=SEED)   # arrivals for rate 1, rescaled below
     unit = [q.arrival for q in base]
     cal = GpuBackend(workers=1)
-    kbars = cal.calibrate()   # the paper's k-bar model, fitted on this GPU (heat_step alone)
+    kbars = cal.calibrate()   # the paper's k-bar model, fitted on this GPU (a batch of one grid)
     cal.close()
 
     def serve(scale):

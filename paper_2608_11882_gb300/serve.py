@@ -135,8 +135,10 @@ class GpuBackend:
         return int(self.torch.cuda.mem_get_info()[0])
 
     def calibrate(self, edges=(96, 160, 256), steps=40) -> dict:
-        """k-bar per arithmetic from heat_step alone on this device (CUDA events
-        around `steps` steps of an edge^3 grid, one warm-up pass each)."""
+        """k-bar per arithmetic of the kernel the server steps requests with: a batch
+        of one edge^3 grid alone on this device (CUDA events around `steps` steps,
+        one warm-up pass each).  heat_step would not do: it takes small grids
+        through another kernel."""
         torch = self.torch
         out = {}
         for dt in ("f64", "f32"):
@@ -144,11 +146,13 @@ class GpuBackend:
             for n in edges:
                 with self.pkg.Heat(n, n, n, 0.1, dtype=dt, stream=self.stream, tdepth=1) as h:
                     h.upload(np.random.default_rng(n).uniform(-1, 1, (n, n, n)).astype(h.np_dtype))
-                    h.step(4)
-                    e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-                    e0.record(self.stream)
-                    h.step(steps)
-                    e1.record(self.stream)
+                    self.heat_advance([h], [4])
+                    with self.pkg.HeatBatch([h], [steps], stream=self.stream) as b:
+                        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+                        e0.record(self.stream)
+                        b.run(use_graph=False)
+                        e1.record(self.stream)
+                        b.wait()
                     e1.synchronize()
                     samples.append((n ** 3, steps, e0.elapsed_time(e1) * 1e-3))
             out[dt] = kbar(samples)
