@@ -15,6 +15,7 @@
 // double once -- and spends two or three FP64 instructions per update, where
 // the formula takes 23.  Fields outside that form's exponent range use the
 // formula itself.
+#include <algorithm>
 #include <cmath>
 
 #include "heat_common.cuh"
@@ -419,7 +420,9 @@ int vk_launch(const VkCall& c)
 {
     const HeatGeom& g = *c.g;
     if (c.kend <= c.kbeg) return HS_OK;
-    const int nchunks = (c.kend - c.kbeg + c.kchunk - 1) / c.kchunk;
+    const int planes = c.kend - c.kbeg;
+    const int kchunk = std::max(c.kchunk, (planes + 65534) / 65535);   // a launch holds 65535 chunks
+    const int nchunks = (planes + kchunk - 1) / kchunk;
     const dim3 block(kVkBX, kVkBY, 1);
     const unsigned by = (g.ny + kVkBY - 1) / kVkBY;
     if (c.f64) {
@@ -446,13 +449,13 @@ int vk_launch(const VkCall& c)
         }();
         HS_TRY_CUDA(configured, "heat: variable-kappa kernel smem attribute");
         const dim3 grid((g.nx + kVkTW - 1) / kVkTW, by, nchunks);
-        kern<<<grid, block, kVkSmem, c.stream>>>(*c.umap, *c.kmap, *c.fmap, (double*)c.dst, g, B, c.kbeg, c.kend, c.kchunk,
+        kern<<<grid, block, kVkSmem, c.stream>>>(*c.umap, *c.kmap, *c.fmap, (double*)c.dst, g, B, c.kbeg, c.kend, kchunk,
                                                  c.fx, c.m3, c.err);
     } else {
         const dim3 grid((g.nx + 4 * kVkBX - 1) / (4 * kVkBX), by, nchunks);
         k_vk_f4<<<grid, block, 0, c.stream>>>((const float*)c.src, (float*)c.dst, (const float*)c.kap,
                                                        (const float*)c.fdt, g, (float)c.bx, (float)c.by, (float)c.bz,
-                                                       c.kbeg, c.kend, c.kchunk);
+                                                       c.kbeg, c.kend, kchunk);
     }
     HS_CHECK_LAUNCH("heat variable-kappa kernel");
     return HS_OK;
