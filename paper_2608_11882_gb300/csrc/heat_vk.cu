@@ -78,6 +78,7 @@ struct VkBeta {
     double bx, by, bz;        // dt / (2 h_d^2)
     double b;                 // the largest
     int wh[3], wl[3];         // beta_d / b times 2^62, as xs_mulhi3 takes it
+    long long low;            // what the three products fall short by on average
     int exact;                // every kappa is in [0.5, 1)
 };
 
@@ -221,7 +222,8 @@ __device__ __forceinline__ unsigned vk_march(const CUtensorMap* umap, const CUte
                     const long long dz = fa - fb[q];
                     fb[q] = fa;
                     const long long L = CUBIC ? dx + dy + dz
-                                              : xs_mulhi3(dx << 2, B.wh[0], B.wl[0]) + xs_mulhi3(dy << 2, B.wh[1], B.wl[1]) +
+                                              : B.low + xs_mulhi3(dx << 2, B.wh[0], B.wl[0]) +
+                                                    xs_mulhi3(dy << 2, B.wh[1], B.wl[1]) +
                                                     xs_mulhi3(dz << 2, B.wh[2], B.wl[2]);
                     const double uf = __dadd_rn(uc[q], q ? f.y : f.x);
                     w[q] = q == 0 ? xs_apply<true>(uf, L, B.b, r2, emax) : xs_apply<false>(uf, L, B.b, r2, emax);
@@ -432,11 +434,18 @@ int vk_launch(const VkCall& c)
         B.bz = c.bz;
         B.b = std::fmax(c.bx, std::fmax(c.by, c.bz));
         const double axis[3] = {c.bx, c.by, c.bz};
+        // xs_mulhi3 rounds two partial products down and leaves out the third, in the
+        // mean one unit and wl / 2^33; with the largest beta's 2^62 it is exact here.
+        // Fluxes round down alike and their bias cancels in a face's difference, this
+        // one would add up from step to step.
+        double low = 0.0;
         for (int d = 0; d < 3; ++d) {
             const long long w = B.b > 0.0 ? std::llrint(std::ldexp(axis[d] / B.b, 62)) : 0ll;
             B.wl[d] = (int)(unsigned)w;
             B.wh[d] = (int)((w - B.wl[d]) >> 32);
+            if (w != 0 && w != 1ll << 62) low += 1.0 + std::ldexp((double)B.wl[d], -33);
         }
+        B.low = std::llrint(low);
         B.exact = c.exact;
         const bool cubic = c.bx == c.by && c.by == c.bz;
         auto kern = cubic ? k_vk_xs<true> : k_vk_xs<false>;
