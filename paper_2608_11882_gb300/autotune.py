@@ -131,7 +131,10 @@ def _flags(pkg, arith):
 
 
 def _gpu_timer(arith: str, shape, depth: int, kc_factor: float = 1.0, steps: int = 24) -> float:
-    """Seconds per step of heat_step on the current device (CUDA events)."""
+    """Seconds per step of heat_step on the current device (CUDA events); infinite
+    for another chunk length where heat_step takes all steps in one launch, which
+    has no chunks: the choice would be one of noise, and grids of the same class
+    that do have chunks would be given it."""
     import numpy as np
     import torch
 
@@ -145,7 +148,10 @@ def _gpu_timer(arith: str, shape, depth: int, kc_factor: float = 1.0, steps: int
             lib_kc = native.heat_get_kchunk(h.handle)
             native.heat_set_kchunk(h.handle, max(4, int(round(lib_kc * kc_factor))))
         h.upload(u0.astype(h.np_dtype))
+        before = native.launch_count()
         h.step(depth * 2)   # warm-up
+        if depth == 1 and kc_factor != 1.0 and native.launch_count() - before == 1:
+            return float("inf")
         e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
         s = torch.cuda.current_stream()
         e0.record(s)
