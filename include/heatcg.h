@@ -90,10 +90,11 @@ extern "C" {
  * on the device beside u, as in the paper's 1-GPU Baseline.  For HS_F64 each
  * face's flux (kappa + kappa_nb)(u_nb - u) is formed in integers on the field's
  * fixed-point scale (its largest exponent, tracked on the device as for the
- * default FP64 arithmetic), the six are summed exactly and rounded once: error
- * below 30 * 2^-57 max|u| beta plus a few roundings per step; fields outside
- * [2^-903, 2^1007] in magnitude
- * step in FP64 arithmetic.  HS_F64 or
+ * default FP64 arithmetic), to within 2.5 units of 2^-57 max|u|.  On
+ * a cubic grid the six are summed exactly and rounded once; elsewhere each axis's
+ * two are summed and scaled by beta_d / beta_max to within another 2.5 units first.
+ * The error stays below 30 * 2^-57 max|u| beta plus a few roundings per step;
+ * fields outside [2^-903, 2^1007] in magnitude step in FP64 arithmetic.  HS_F64 or
  * HS_F32; excludes HS_FIXED64, HS_EXACT_ROUNDING, HS_SCHED_FULL and tdepth > 1;
  * cannot join a heat batch. */
 #define HS_VARKAPPA         0x10u
@@ -124,9 +125,10 @@ typedef struct {
     int32_t  dtype;        /* HS_F64 or HS_F32: storage and arithmetic type   */
     int32_t  tdepth;       /* time steps per pass over HBM: 0 = library choice
                               (2 for HS_F32 without HS_VARKAPPA or
-                              HS_SCHED_FULL, else 1), 1 = the Interior + Boundary
-                              kernels every step, or 2, 3, 4 = temporal
-                              blocking (see heat_step)                     */
+                              HS_SCHED_FULL, else 1), 1 = one step per pass
+                              (Interior + Boundary kernels, or for small grids
+                              one launch for many steps), or 2, 3, 4 =
+                              temporal blocking (see heat_step)            */
     void*    stream;       /* cudaStream_t for all work of this handle        */
     void*    dev_buf0;     /* optional caller-owned device buffers for the two
                               time levels (for example torch allocations):
@@ -231,16 +233,18 @@ int heat_read(hs_heat_t h, void* dst, int dst_is_device);
 /* Steps applied since the last heat_upload. */
 int heat_steps_done(hs_heat_t h, int64_t* steps);
 
-/* The temporal depth the handle runs with (tdepth resolved: 1 = the Interior
- * + Boundary kernels every step, L >= 2 = L steps per pass, or four where the
- * library chose the depth and that is faster). */
+/* The temporal depth the handle runs with (tdepth resolved: 1 = one step per
+ * pass, L >= 2 = L steps per pass, or four where the library chose the depth and
+ * that is faster).  Small grids may take all steps in one launch at either
+ * (see heat_step). */
 int heat_get_tdepth(hs_heat_t h, int32_t* tdepth);
 
 /* Planes each block of the one-step Interior kernel takes (the k-chunk of
  * Section 6.1's k-split, applied within one GPU): planes >= 1 sets it (capped
  * at the interior's nz - 2), 0 restores the library's choice.  It changes
  * speed only -- every point is computed the same way -- and does not apply to
- * temporally blocked passes.  heat_get_kchunk reports the value in use. */
+ * temporally blocked passes, nor to the small grids that heat_step advances in
+ * one launch (heat_interior there still takes it).  heat_get_kchunk reports the value in use. */
 int heat_set_kchunk(hs_heat_t h, int32_t planes);
 int heat_get_kchunk(hs_heat_t h, int32_t* planes);
 
@@ -424,10 +428,11 @@ int cg_create_mixed(hs_cg_t* out, const hs_op* A, const hs_cg_mixed_opts* opts, 
 int cg_destroy(hs_cg_t c);
 
 /* Batched CG: n independent systems (each its own operator, device b and x)
- * solved together -- three kernel launches per iteration for the whole batch.
- * Each system uses the row partition and reduction order its own cg_run
- * would use, so its results equal solving it alone bit for bit; a system
- * stops when it reaches rtol or max_iter while the others go on.  infos (may
+ * solved together -- the stencil systems of 2^14 to 2^22 unknowns whole in one
+ * launch, the others with three to five launches per iteration for all of them.
+ * Each system keeps the partition and the order of sums its own cg_run has, so
+ * its results equal solving it alone bit for bit; a system stops when it reaches
+ * rtol or max_iter while the others go on.  infos (may
  * be NULL) receives one hs_cg_info per system.  Returns HS_OK when every
  * system converged, HS_ENOCONV if any did not (x and infos filled anyway).
  * Operators must be device memory and outlive the batch. */
@@ -454,7 +459,7 @@ int cg_solve(const hs_op* A, const void* b, void* x, double rtol, int32_t max_it
  * Same arguments, same kernels and the same results as cg_solve; it calls no
  * cudaMalloc, cudaFree, cudaMallocHost or other allocating routine.  The
  * solver's scratch (r, p, q, reduction partials, device scalars) lives in one
- * fixed array of about 50 MB inside the library, which every GPU that loads
+ * fixed array of about 54 MB inside the library, which every GPU that loads
  * the library holds until the process exits.
  *   - A's arrays, b and x must be device memory (A->host == 0).
  *   - n > HS_NOALLOC_MAX_N is rejected with HS_EINVAL before any work.

@@ -1,6 +1,6 @@
 // Conjugate gradients on the 7-point Dirichlet Laplacian (Section 7.5):
-// SpMV fused with the p.q dot product, the x/r update fused with r.r, the
-// p update, deterministic grid reductions, and the cg_* / op_apply entry
+// SpMV fused with the p.q dot product, the r update fused with r.r, the p update,
+// x with one or the other, deterministic grid reductions, and the cg_* / op_apply entry
 // points of the C ABI.
 //
 // CG in the textbook form (unpreconditioned, FP64; the matrix-free SpMV forms
@@ -739,7 +739,7 @@ constexpr size_t kNoAllocPartials = 2 * (size_t)(kNoAllocMaxGrid > kCgSmallMaxBr
 constexpr size_t kNoAllocVector = (size_t)(kNoAllocMaxN + kNoAllocMaxN / kCgSmallMinNx);
 constexpr size_t kNoAllocDoubles = 3 * kNoAllocVector + kNoAllocPartials + kNoAllocCtlDoubles;
 
-// About 50 MB.  Every GPU that loads this library holds it until the process exits.
+// 53.5 MB.  Every GPU that loads this library holds it until the process exits.
 static __device__ __align__(256) double g_noalloc_scratch[kNoAllocDoubles];
 
 // Device address of g_noalloc_scratch per device (host code may not use the

@@ -1,8 +1,10 @@
 // Batched CG: many independent systems A_s x_s = b_s (7-point Laplacians of
-// different grids, matrix-free or CSR) solved together, three kernel launches
-// per iteration for the whole batch instead of three per system.
+// different grids, matrix-free or CSR) solved together.  Stencil systems of 2^14
+// to 2^22 unknowns go through one launch for whole solves (cg_small.cu), the
+// others through an update, a direction and up to three SpMV launches (one per
+// kind present) per iteration for all of them.
 //
-// Each system gets the same number of blocks and the same grid-stride row
+// Each of those others gets the same number of blocks and the same grid-stride row
 // partition as its own cg_run would use, its own reduction partials, ticket
 // and device scalars, so its iterates -- and results -- equal a solve of it
 // alone bit for bit.  Systems that have converged (or hit max_iter) stop at

@@ -22,8 +22,8 @@
 // sums and the halo loads), 96^3 25.2, 128^3 44.9 (start: 33.8, 49.2, 73.2); 64
 // systems of 22.9 M unknowns in all 149 ms, start 429: 1.8 x what their vectors'
 // 80 bytes per row take at the copy rate, the FP64 pipe 55% and DRAM 43% busy --
-// each phase waits on its loads part of the time.  Four blocks per SM (64
-// registers, spilling) took 155 ms.
+// each phase waits on its loads part of the time.  Three blocks per SM (80
+// registers, 152 bytes of spill); four (64 registers, more spill) took 155 ms.
 //
 // Vectors change hands between SMs from phase to phase, so they are read with
 // ld.global.cg (L2), never through L1.

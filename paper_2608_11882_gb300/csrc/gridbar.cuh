@@ -9,9 +9,9 @@
 // when some block still holds the previous value and none exceeds it, the
 // arrival word alone gives the result.  Blocks with another value also fold it
 // into a second word, which is read only when the first does not decide.
-// Three sets of words are used in turn; block 0 clears the next set before it arrives, when every block has left it.  (All blocks reading all
-// blocks' values instead of counting measured 3.6 us more per phase at 128
-// blocks.)
+// Three sets of words are used in turn; block 0 clears the next set before it
+// arrives, when every block has left it.  (All blocks reading all blocks' values
+// instead of counting measured 3.6 us more per phase at 128 blocks.)
 //
 // Every wait is bounded: one that runs out sets *err, which ends the others.
 #pragma once

@@ -308,7 +308,6 @@ struct hs_heat {
     int kchunk;        // planes per Interior-kernel block
     int tdepth;        // steps per pass of the temporally blocked kernel (1: Interior + Boundary)
     bool deep;         // the library chose the depth, and passes of four steps are faster here
-    int kc_tb;         // k-planes per block of the temporally blocked kernel
     CUtensorMap maps[2];   // TMA maps of the two buffers (temporal blocking)
     CUtensorMap smaps[2];  // TMA maps of the two buffers (streaming Interior kernel)
     uint32_t tbox[2];      // box of maps[]
@@ -1265,8 +1264,8 @@ int heat_read(hs_heat_t h, void* dst, int dst_is_device)
                               "the block's loads in flight did not complete in time; the field is not "
                               "valid and the CUDA context should be treated as suspect");
     if (err)
-        return fail(HS_ETIMEOUT, "heat_read: a bounded wait inside a TMA-staged heat kernel ran out; "
-                                 "the field is not valid");
+        return fail(HS_ETIMEOUT, "heat_read: a bounded wait inside a heat kernel (for a TMA load, or at the "
+                                 "multi-step kernel's barrier) ran out; the field is not valid");
     if (h->arith == A_FX64) {
         FxState st;
         HS_TRY_CUDA(cudaMemcpyAsync(&st, h->fx, sizeof(st), cudaMemcpyDeviceToHost, h->stream),

@@ -14,9 +14,9 @@
 // with several, by instruction issue, the z halo converted twice per four
 // planes.  At least two blocks per SM, every block resident, so that one loads
 // while the other computes (held to three the kernel took 17.7 us instead of
-// 15.4 per FP64 step of 191 x 101 x 150).  The per-point arithmetic is that of the other heat kernels, so
-// results match them bit for bit, and the whole grid -- Interior and Boundary
-// planes -- is one step's work.
+// 15.4 per FP64 step of 191 x 101 x 150).  The per-point arithmetic is that of the
+// other heat kernels, so results match them bit for bit, and the whole grid --
+// Interior and Boundary planes -- is one step's work.
 #include <algorithm>
 
 #include "gridbar.cuh"

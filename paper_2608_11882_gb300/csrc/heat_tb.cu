@@ -10,12 +10,12 @@
 // thread keeps level t-1's values at k-1 and k in registers and receives the
 // value at k+1 from the level just computed; the x/y neighbours come from
 // shared planes per level, in FP32 with a warp per row the x neighbours by lane
-// shuffle (the neighbour between a thread's two rows from its own registers).  Only level L reaches HBM, so a pass moves
-// (8 or 16 bytes)/L per point-step plus the halo.  Positions outside the
-// interior and planes outside [0, nz) are the Dirichlet zeros at every level;
-// level 0 reads them from the zero boundary layer of the padded buffer or from
-// TMA's zero fill beyond it.  Blocks whose every computed point lies inside
-// the interior skip the masks.
+// shuffle (the neighbour between a thread's two rows from its own registers).
+// Only level L reaches HBM, so a pass moves (8 or 16 bytes)/L per point-step plus
+// the halo.  Positions outside the interior and planes outside [0, nz) are the
+// Dirichlet zeros at every level; level 0 reads them from the zero boundary layer
+// of the padded buffer or from TMA's zero fill beyond it.  Blocks whose every
+// computed point lies inside the interior skip the masks.
 //
 // Every mbarrier wait is bounded; a wait that runs out sets the handle's
 // device error word (read as HS_ETIMEOUT by heat_read), waits (again bounded)
@@ -77,10 +77,10 @@ struct TbShape {
     // Shared planes a level keeps: two in turn, or in FP32 as many as the ring has
     // stages, in the ring's slots (constants there; FIXED64 at depth 4 loses 3%)
     static constexpr int LEV = std::is_same<T, float>::value ? 3 : 2;
-    // FP32 warp rows: 16 (64 registers, two blocks of 16 warps per SM at depth 2);
-    // the halo rows weigh less than with 12: 512^3 125.0 -> 123.1 us per step,
-    // 1000^3 828 -> 767, at depth 4 143 -> 128.  Wider types, and rows of 34
-    // threads, would spill.
+    // FP32 warp rows: 16 (64 registers, 32 bytes of spill at depth 2, two blocks of 16
+    // warps per SM); the halo rows weigh less than with 12: 512^3 125.0 -> 123.1 us
+    // per step, 1000^3 828 -> 767, at depth 4 143 -> 128.  Rows of 34 threads would
+    // spill 140 to 336 bytes, FIXED64 12; FP64, bound by its pipe, keeps 12 with it.
     static constexpr int RR = std::is_same<T, float>::value && W == 32 ? 16 : 12;
     static constexpr int REG = RR * RT;
     static constexpr int TY = REG - 2 * L;
@@ -466,7 +466,8 @@ void tb_tile(int arith, int L, int nx, int* tx, int* ty)
 
 // Per step, depth 2 / depth 4: 32-thread rows 220^3 15.6 / 11.8 us, 333^3 38.0 /
 // 32.9, 512^3 121.9 / 112.3, 640^3 211 / 211, 1000^3 764 / 697; 34-thread rows
-// (the depth-4 pass spills with their blocks) 256^3 21.3 / 24.1, 384^3 56.5 / 64.7.
+// (12 of them: 24 rows of a region leave 16 at depth 4, 20 at depth 2) 256^3 21.3 /
+// 24.1, 384^3 56.5 / 64.7.
 bool tb_deep(int arith, int nx)
 {
     return arith == A_F32 && tb_row_threads(arith, nx) == 32;

@@ -71,13 +71,14 @@ __device__ __forceinline__ long long xs_fix(long long bits, int emax)
     return q;
 }
 
-// x 2^(emax - 1080) rounded to the nearest double, ties to even (|x| < 2^62,
+// x 2^(emax - 1080) rounded to the nearest double, ties to even (|x| < 2^63: the
+// six-point sums stay below 2^62, the variable-coefficient ones below 1.43 2^62;
 // xs_emax_lo <= emax <= kXsEmaxHi, so the result is a normal number or zero).
 __device__ __forceinline__ double xs_unfix(long long x, int emax)
 {
     const unsigned long long s = (unsigned long long)(x >> 63);
     const unsigned long long a = ((unsigned long long)x ^ s) - s;
-    const int lz = __clzll((long long)a);                       // >= 2; 64 for a = 0
+    const int lz = __clzll((long long)a);                       // >= 1; 64 for a = 0
     unsigned long long n;                                       // leading one at bit 62
     asm("shl.b64 %0, %1, %2;" : "=l"(n) : "l"(a), "r"(lz - 1));
     const unsigned long long q = (n + 0x1ffull + ((n >> 10) & 1ull)) >> 10;   // 2^52 <= q <= 2^53, or 0
