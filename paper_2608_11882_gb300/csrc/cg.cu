@@ -472,13 +472,23 @@ int cg_create_vectors(hs_cg_t* out, const hs_op* A, void* stream, bool need_p)
         two = false;
     }
     if (!two) CG_ALLOC(c->arena, s_ctl + s_part + (need_p ? 3 : 2) * s_vec);
-    c->ctl = (char*)c->arena;
+    // Vectors first, then what every block polls and counts on.  With the control
+    // words and partials in front, the placement of the same few lines made small
+    // solves 9% slower on one GPU and 5% faster on another (25^3: 1586 -> 1738 us,
+    // 1645 -> 1569); in this order they stay within 1% of separate allocations.
+    char* at = (char*)c->arena;
+    auto take = [&](size_t bytes) {
+        char* const a = at;
+        at += bytes;
+        return a;
+    };
+    c->r = (double*)take(s_vec);
+    c->p = need_p ? (double*)take(s_vec) : nullptr;
+    c->q = (double*)take(s_vec);
+    c->p2 = two ? (double*)take(s_vec) : nullptr;
+    c->partials = (double*)take(s_part);
+    c->ctl = take(s_ctl);
     c->S = &((CgSmallCtl*)c->ctl)->S;
-    c->partials = (double*)(c->ctl + s_ctl);
-    c->r = (double*)(c->ctl + s_ctl + s_part);
-    c->q = (double*)(c->ctl + s_ctl + s_part + s_vec);
-    c->p = need_p ? (double*)(c->ctl + s_ctl + s_part + 2 * s_vec) : nullptr;
-    c->p2 = two ? (double*)(c->ctl + s_ctl + s_part + 3 * s_vec) : nullptr;
     // the host mirror of the scalars: ordinary memory (pinned memory would
     // cost a device-wide synchronisation to allocate and to free)
     c->S_host = new (std::nothrow) CgScalars();
