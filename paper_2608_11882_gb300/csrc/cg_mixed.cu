@@ -46,7 +46,7 @@ struct MxScalars {
     int32_t first;        // 1 until ||b|| has been computed
     int32_t inner;        // iterations of the current inner solve
     int32_t pad;
-    double alpha2[2];     // alpha of its iteration i in slot i % 2
+    double alpha0;        // alpha of its last even iteration
 };
 
 struct OpDev32 {
@@ -490,10 +490,7 @@ __global__ void __launch_bounds__(kCgBlock, 1)
         if (!(tot > 0.0))
             S->inner_done = 2;
         else
-        {
             S->alpha = S->rho / tot;
-            S->alpha2[S->inner & 1] = S->alpha;
-        }
     }
 }
 
@@ -555,7 +552,9 @@ __global__ void __launch_bounds__(kCgBlock)
 // alpha0 p0, then d += alpha p, p0 the direction before p), so d is read and
 // written every second iteration: 20 bytes per row on average instead of 24.
 // What the last, even iteration of an inner solve leaves is added by
-// k_mx_correct.  Four blocks per SM with the loop unrolled by four: 127.3 us per
+// k_mx_correct.  The even update keeps its alpha, not the SpMV, whose end every
+// iteration waits for: 32^3 3014 -> 2954 us, where the update that took d every
+// time had 2982.  Four blocks per SM with the loop unrolled by four: 127.3 us per
 // iteration at 256^3 and 445 at 400^3, against 130.7 and 511 with eight (and the
 // update that took d every time: 138.9 and 544).
 template <bool ODD>
@@ -566,7 +565,7 @@ __global__ void __launch_bounds__(kCgBlock)
     grid_dependency_wait();
     if (*(volatile int32_t*)&S->inner_done) return;
     __shared__ double sh[kCgBlock / 32];
-    const float alpha = (float)S->alpha, alpha0 = ODD ? (float)S->alpha2[0] : 0.0f;
+    const float alpha = (float)S->alpha, alpha0 = ODD ? (float)S->alpha0 : 0.0f;
     Acc32 rr;
     // the vectors hold a multiple of four values and start aligned (nx % 4 == 0)
     const int64_t t0 = (int64_t)blockIdx.x * kCgBlock + threadIdx.x, stride = (int64_t)gridDim.x * kCgBlock;
@@ -597,6 +596,7 @@ __global__ void __launch_bounds__(kCgBlock)
     const double rho_new = sum_partials(partials, gridDim.x, sh);
     if (threadIdx.x == 0) {
         S->ticket = 0;
+        if (!ODD) S->alpha0 = S->alpha;
         S->iters += 1;
         S->inner += 1;
         if (rho_new <= S->inner_stop) {
@@ -636,7 +636,7 @@ __global__ void __launch_bounds__(kCgBlock)
                  const MxScalars* S)
 {
     const bool left = p != nullptr && (S->inner & 1) != 0;
-    const float alpha = (float)S->alpha2[0];
+    const float alpha = (float)S->alpha0;
     for (int64_t t = (int64_t)blockIdx.x * kCgBlock + threadIdx.x; t < n;
          t += (int64_t)gridDim.x * kCgBlock)
         x[t] += (double)(left ? __fmaf_rn(alpha, p[t], d[t]) : d[t]);
