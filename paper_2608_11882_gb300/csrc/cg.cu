@@ -114,7 +114,9 @@ __global__ void __launch_bounds__(kCgBlock)
 }
 
 // The matrix-free SpMV staged by loads (SP_STAGED), fused with p.q: one block
-// of kSpBlock threads per share (spmv_shares of the solve's block count).
+// of kSpBlock threads per share (spmv_shares of the solve's block count).  It
+// spills 28 bytes with xs_fix's shorter form and is the faster for that form all
+// the same (163^3 50.5 ms per solve, 50.8 without).
 __global__ void __launch_bounds__(kSpBlock, kSpMinBlocks)
     k_cg_spmv_staged(OpDev A, const double* __restrict__ p, double* __restrict__ q, double* partials,
                      CgScalars* S)

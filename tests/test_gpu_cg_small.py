@@ -126,3 +126,23 @@ def test_overflowing_pq_ends_at_max_iter(pkg, shape):
             assert infos[1 - k]["converged"] and torch.equal(xs[1 - k], xo)
             xs, infos = cb.run(bs, rtol=1e-8, max_iter=its)
             assert [i["iters"] for i in infos] == [its, its] and torch.equal(xs[k], x0)
+
+
+@pytest.mark.parametrize("shape", [(32, 32, 64), (128, 128, 128), (12, 20, 18)])
+@pytest.mark.parametrize("bad", [np.inf, np.nan])
+def test_right_hand_side_that_is_not_finite(pkg, shape, bad):
+    """A breakdown, alone and in a batch, and the context solves on."""
+    nz, ny, nx = shape
+    b = cg_rhs(nx * ny * nz, seed=3)
+    poisoned = b.copy()
+    poisoned[nx * ny + 5] = bad
+    op, other = pkg.Operator.stencil(nx, ny, nz), pkg.Operator.stencil(30, 28, 26)
+    bo = dev(cg_rhs(30 * 28 * 26, seed=1))
+    with pkg.CG(op) as cg, pkg.CGBatch([other, op]) as cb:
+        with pytest.raises(Exception, match="breakdown"):
+            cg.run(dev(poisoned), max_iter=40)
+        with pytest.raises(Exception, match="breakdown in system 1"):
+            cb.run([bo, dev(poisoned)], max_iter=40)
+        x, info = cg.run(dev(b), rtol=1e-6, max_iter=2000)
+        xs, infos = cb.run([bo, dev(b)], rtol=1e-6, max_iter=2000)
+    assert info["converged"] and infos[0]["converged"] and np.array_equal(xs[1].cpu().numpy(), x.cpu().numpy())
